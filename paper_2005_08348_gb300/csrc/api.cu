@@ -699,6 +699,7 @@ const char *fill_force_field(const mdas_system_desc *d, double shrink, Params &P
     P.rc2f_lo = (float)(P.rc2 * (1.0 - 1e-5));
     P.krf2f = (float)(2.0 * P.krf);
     P.kb = d->kb; P.b0 = d->b0; P.kth = d->ktheta; P.cos0 = std::cos(d->theta0_deg * M_PI / 180.0);
+    P.kbf = (float)P.kb; P.b0f = (float)P.b0; P.kthf = (float)P.kth; P.cos0f = (float)P.cos0;
     P.precision = d->precision;
     const double rc6 = std::pow(d->rc, 6);
     for (int a = 0; a < nbt; ++a)
@@ -837,7 +838,7 @@ mdas_status mdas_create_system(const mdas_system_desc *d, mdas_system **out) {
         P.n_lcells = ld.n_lcells;
         for (int k = 0; k < 3; ++k) P.pc_lmin[k] = std::max(P.nc[k] * d->rc, ld.ln[k] * P.rl);
         P.lcapc = ld.lcapc;
-        if (P.lcapc > NLB_BEADS * 32767) {     // a cell's build tasks are counted in 15 bits
+        if (P.lcapc > NLB_FEW * 32767) {     // a cell's build tasks are counted in 15 bits
             delete s;
             return fail(nullptr, MDAS_ERR_INVALID_ARG, "create: too many beads in a list-build cell");
         }
@@ -898,7 +899,7 @@ mdas_status mdas_create_system(const mdas_system_desc *d, mdas_system **out) {
         {(void **)&H.lcell, 8ull * P.n_lcells}, {(void **)&H.lid, 4ull * n}, {(void **)&H.lk, 4ull * n},
         {(void **)&H.lpos, 32ull * n}, {(void **)&H.xref, 16ull * n}, {(void **)&H.nl_n, 4ull * NL_LANES_MAX * n},
         {(void **)&H.nl, 4ull * (size_t)P.lcap * P.npad}, {(void **)&H.bslot, 4ull * NL_PART * n},
-        {(void **)&H.btask, 8ull * (n / NLB_BEADS + P.n_lcells + 1)},
+        {(void **)&H.btask, 8ull * (n / NLB_FEW + P.n_lcells + 1)},
         {(void **)&H.tmark, 8ull * P.mark_words},
     };
     size_t total = 0;
@@ -1955,7 +1956,7 @@ size_t arena_estimate(const mdas_system_desc *d) {
     const ListDims ld = list_dims(d, shrink);
     t += 12ull * ld.n_lcells + 4ull * ld.n_lcells * ld.lcapc + 4 * n + 4 * n + 32 * n + 16 * n + 4ull * NL_LANES_MAX * n +
          4ull * ld.lcap * ld.npad + 4ull * NL_PART * n + 8ull * ((n + NL_BEADS_MIN - 1) / NL_BEADS_MIN / 32 + 1) +
-         8ull * (n / NLB_BEADS + ld.n_lcells + 1);
+         8ull * (n / NLB_FEW + ld.n_lcells + 1);
     return t + 52 * 256;
 }
 

@@ -26,10 +26,11 @@ constexpr int NL_LANES_MAX = 4;        // the most list columns per bead of any 
 constexpr int NL_BEADS_MIN = NL_BLOCK / NL_LANES_MAX;   // beads of the smallest step item
 __host__ __device__ constexpr bool nl_lanes_ok(int g) { return g == 2 || g == 4; }
 constexpr int NL_PART = 8;             // bonded partners per bead at most
-constexpr int NLB_BEADS = 8;           // beads of one list-build task (one warp)
+constexpr int NLB_BEADS = 8;           // beads of one list-build task (one warp),
+constexpr int NLB_FEW = 2;             // and where the tasks would leave most warps idle
 constexpr int NL_BUILD_BLOCKS = 152 * 8;   // blocks of the list-build kernel (separate launches)
-// list-build tasks of a cell with the given number of beads
-__host__ __device__ constexpr int nl_build_tasks(int beads) { return (beads + NLB_BEADS - 1) / NLB_BEADS; }
+// list-build tasks of a cell with the given number of beads, at most run per task
+__host__ __device__ constexpr int nl_build_tasks(int beads, int run) { return (beads + run - 1) / run; }
 constexpr int CELLS_PER_SORT_BLOCK = 4;
 constexpr int LOG_CAP = 65536;         // trial records kept per system
 constexpr int MAX_ROUND_TRIALS = 1024; // trials per batched swap evaluation
@@ -75,7 +76,11 @@ __host__ __device__ inline int meta_lip(uint32_t m) { return (int)(m >> 12) - 1;
 
 // Parameters of one system (device memory).  Kernels read them; only the
 // pressure coupling changes the box fields, between launches (k_pcouple).
-struct Params {
+//
+// ParamsHot: the scalars and the lipid topology, which the step items copy to
+// shared memory (they do not change during a launch, and the L1 cache is
+// invalidated at every grid barrier); Params adds the pair tables.
+struct ParamsHot {
     int n, n_lip, bpl, n_bt, n_lt, n_lipid_beads;
     int nc[3], n_cells, capc;          // cells per edge, cells, bead capacity of a cell
     double box[3], qs[3], qdt[3];      // qs = L/2^32; qdt = dt 2^32 / L
@@ -90,6 +95,7 @@ struct Params {
     int nf[2];
     double ktarget[2];
     double kb, b0, kth, cos0;
+    float kbf, b0f, kthf, cos0f;       // the same in single precision
     uint32_t key0, key1;
     int precision;
     uint32_t rcu[3];                   // rc in fixed-point units per axis (rounded up)
@@ -106,15 +112,6 @@ struct Params {
     double rl, rl2;
     float rl2f;                        // rl^2 rounded up (build cull)
     float dmax2f;                      // squared displacement since the build that invalidates the list
-    int8_t npart[16], part[16][NL_PART];   // bonded partners (local indices) of local index k
-    int8_t pidx[16][16];               // local index -> slot in part[k], -1 if not a partner
-    // pair tables [ti*16 + tj]; qq includes f / eps_r
-    double c12[256], c6[256], qq[256], ush[256];
-    float f12f[256], f6f[256], qqf[256];   // 12 C12, 6 C6, f qi qj / eps_r
-    uint8_t lbt[256];                  // [lipid type * 16 + k] -> bead type
-    uint16_t excl[16];                 // excluded partners of local index k (1-2 bonds)
-    int8_t nbond[16], bpart[16][4];
-    int8_t nang[16], ang[16][8][3];    // angles containing local index k
     // semi-isotropic Parrinello-Rahman pressure coupling (Sec. 3), on when pc_nst > 0
     int pc_nst;                        // MD steps per box update
     double pc_pref, pc_wc;             // bar; 4 pi^2 beta / (3 tau_p^2) (the inverse barostat mass times L_max)
@@ -123,6 +120,18 @@ struct Params {
     double dtm_pc[3];                  // dt (dL/dt) / L of the current interval (the particles' -M v term)
     float dtm_pcf[3];
     double pres[3];                    // pressure tensor diagonal of the last box update, bar
+    int8_t npart[16], part[16][NL_PART];   // bonded partners (local indices) of local index k
+    int8_t pidx[16][16];               // local index -> slot in part[k], -1 if not a partner
+    int8_t nbond[16], bpart[16][4];
+    int8_t nang[16], ang[16][8][3];    // angles containing local index k
+};
+
+struct Params : ParamsHot {
+    // pair tables [ti*16 + tj]; qq includes f / eps_r
+    double c12[256], c6[256], qq[256], ush[256];
+    float f12f[256], f6f[256], qqf[256];   // 12 C12, 6 C6, f qi qj / eps_r
+    uint8_t lbt[256];                  // [lipid type * 16 + k] -> bead type
+    uint16_t excl[16];                 // excluded partners of local index k (1-2 bonds)
 };
 
 constexpr double BAR_PER_KJ_MOL_NM3 = 16.6053906717;   // 10^3 / N_A / 10^-27 m^3 / 10^5 Pa, N_A = 6.02214076e23
@@ -246,12 +255,23 @@ struct SysDev {
     uint4 *lpos;                       // [2 n] positions in list order, two buffers
     uint4 *xref;                       // [n] positions when the list was built
     int *nl_n;                         // [n * G] entries in each column of each bead's list
-    int *nl;                           // row r of column g of bead k at [r * npad * G + k * G + g]
+    int *nl;                           // pair list: row r of column g of bead k at nl_at<G>(npad, k, r, g)
     int *bslot;                        // [n * NL_PART] list indices of the bonded partners
-    int2 *btask;                       // [n / NLB_BEADS + n_lcells + 1] list-build tasks: cell, tasks << 16 | task
+    int2 *btask;                       // [n / NLB_FEW + n_lcells + 1] list-build tasks: cell, tasks << 16 | task
     unsigned *tmark;                   // [2 * mark_words] step items an exchange trial can change, per trial parity
     int n_bead_blocks;
 };
+
+// Place of row r of column g of bead k in the pair list: blocks of 4 rows of
+// every column, so that a lane of the step reads 4 rows at once and a bead's
+// 4 G entries of a block (written one after another by the build) share a
+// 64-byte (G = 4) piece of memory; nl_block_stride entries from block to block.
+template <int G>
+__host__ __device__ inline size_t nl_block_stride(int npad) { return (size_t)npad * (4 * G); }
+template <int G>
+__host__ __device__ inline size_t nl_at(int npad, int k, int r, int g) {
+    return (size_t)(r >> 2) * nl_block_stride<G>(npad) + (size_t)k * (4 * G) + g * 4 + (r & 3);
+}
 
 // ---------------------------------------------------------------- Philox
 // 128 threads of a block that synchronise on their own named barrier `bar`

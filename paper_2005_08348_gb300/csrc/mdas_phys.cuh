@@ -88,7 +88,7 @@ __device__ inline double alpha_for(const SysDev &S, const Params &P, const Count
 // ---------------------------------------------------------- bonded terms
 // Separation r_a - r_b of two beads (exact integer minimum image).
 template <typename Real>
-__device__ __forceinline__ void sep(const Params &P, uint4 a, uint4 b, Real d[3]) {
+__device__ __forceinline__ void sep(const ParamsHot &P, uint4 a, uint4 b, Real d[3]) {
     if (sizeof(Real) == 4) {
         d[0] = (Real)((float)(int)(a.x - b.x) * P.qsf[0]);
         d[1] = (Real)((float)(int)(a.y - b.y) * P.qsf[1]);
@@ -103,25 +103,29 @@ __device__ __forceinline__ void sep(const Params &P, uint4 a, uint4 b, Real d[3]
 // Bonded terms of the bead with local index k at pi: term q < nbond is bond
 // q, the rest are its angles; every stride-th term from `first` is added to f
 // (all of them by default).  get(li) returns the position of the bead with
-// local index li of the same lipid.
+// local index li of the same lipid.  The bonds of a lane's share come before
+// its angles, in two loops, so that the lanes of a bead go through their
+// angles together whatever term they began with.
 // VIR: w also gains this bead's share of the virial sums S_a (the bond's
 // f d_a^2, which its other bead adds as well; twice (r_k - r_vertex)_a F_k,a
 // for an angle that k ends), so that S over all beads counts every term
 // twice, like the pair list.
 template <typename Real, bool VIR = false, class Get>
-__device__ void bonded_force(const Params &P, int k, uint4 pi, Get get, Real f[3], int first = 0, int stride = 1,
-                             Real *w = nullptr) {
+__device__ __forceinline__ void bonded_force(const ParamsHot &P, int k, uint4 pi, Get get, Real f[3], int first = 0,
+                                             int stride = 1, Real *w = nullptr) {
+    constexpr bool F32 = sizeof(Real) == 4;
     const int nb = P.nbond[k], nt = nb + P.nang[k];
-    for (int q = first; q < nt; q += stride) {
-        if (q < nb) {
-            Real d[3];
-            sep<Real>(P, pi, get(P.bpart[k][q]), d);
-            const Real r = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-            const Real fs = -(Real)P.kb * (r - (Real)P.b0) / r;
-            f[0] += fs * d[0]; f[1] += fs * d[1]; f[2] += fs * d[2];
-            if (VIR) { w[0] += fs * d[0] * d[0]; w[1] += fs * d[1] * d[1]; w[2] += fs * d[2] * d[2]; }
-            continue;
-        }
+    int q = first;
+    for (; q < nb; q += stride) {
+        Real d[3];
+        sep<Real>(P, pi, get(P.bpart[k][q]), d);
+        const Real r = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
+        const Real kb = F32 ? (Real)P.kbf : (Real)P.kb, b0 = F32 ? (Real)P.b0f : (Real)P.b0;
+        const Real fs = -kb * (r - b0) / r;
+        f[0] += fs * d[0]; f[1] += fs * d[1]; f[2] += fs * d[2];
+        if (VIR) { w[0] += fs * d[0] * d[0]; w[1] += fs * d[1] * d[1]; w[2] += fs * d[2] * d[2]; }
+    }
+    for (; q < nt; q += stride) {
         const int a = q - nb;
         const int li = P.ang[k][a][0], lj = P.ang[k][a][1], lk = P.ang[k][a][2];
         const uint4 qi = li == k ? pi : get(li);
@@ -134,8 +138,10 @@ __device__ void bonded_force(const Params &P, int k, uint4 pi, Get get, Real f[3
         const Real lb2 = B[0] * B[0] + B[1] * B[1] + B[2] * B[2];
         const Real iab = (Real)1 / sqrt(la2 * lb2);
         const Real cs = (A[0] * B[0] + A[1] * B[1] + A[2] * B[2]) * iab;
-        const Real pre = -(Real)P.kth * (cs - (Real)P.cos0);
+        const Real kth = F32 ? (Real)P.kthf : (Real)P.kth, cos0 = F32 ? (Real)P.cos0f : (Real)P.cos0;
+        const Real pre = -kth * (cs - cos0);
         const Real ia2 = (Real)1 / la2, ib2 = (Real)1 / lb2;
+#pragma unroll
         for (int d = 0; d < 3; ++d) {
             const Real dci = B[d] * iab - cs * A[d] * ia2;
             const Real dck = A[d] * iab - cs * B[d] * ib2;

@@ -158,7 +158,7 @@ __device__ inline void trial_nl_part(const SysDev &S, int p, int par, const Grp 
             if (sm.it_beg[mid] <= f) lo = mid; else hi = mid - 1;
         }
         const int ci = lo / NL_G, q = lo % NL_G, row = f - sm.it_beg[lo];
-        const int kj = MDAS_IDX(*S.c, S.nl[(size_t)row * P.npad * NL_G + (size_t)sm.chg_k[ci] * NL_G + q], P.n);
+        const int kj = MDAS_IDX(*S.c, S.nl[nl_at<NL_G>(P.npad, sm.chg_k[ci], row, q)], P.n);
         if (mark) atomicOr(&mk[kj / NL_BEADS / 32], 1u << (kj / NL_BEADS % 32));
         const uint4 pi = sm.chg_pos[ci], pj = cur[kj];
         const int ix = (int)(pi.x - pj.x), iy = (int)(pi.y - pj.y), iz = (int)(pi.z - pj.z);
@@ -275,7 +275,7 @@ __device__ inline double mdas_work_part(const SysDev &S, int x, int par, const G
         if (oi != ni) {
             const int rows = S.nl_n[(size_t)ki * NL_G + col];
             for (int r = sub; r < rows; r += TPC) {
-                const int kj = MDAS_IDX(*S.c, S.nl[(size_t)r * P.npad * NL_G + (size_t)ki * NL_G + col], P.n);
+                const int kj = MDAS_IDX(*S.c, S.nl[nl_at<NL_G>(P.npad, ki, r, col)], P.n);
                 const uint4 pj = cur[kj];
                 const int ix = (int)(pi.x - pj.x), iy = (int)(pi.y - pj.y), iz = (int)(pi.z - pj.z);
                 const float fx = (float)ix * P.qsf[0], fy = (float)iy * P.qsf[1], fz = (float)iz * P.qsf[2];

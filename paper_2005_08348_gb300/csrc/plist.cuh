@@ -51,6 +51,7 @@
 #pragma once
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "mdas_phys.cuh"
 #include "mdas_trial.cuh"
@@ -68,17 +69,47 @@ __device__ __forceinline__ int lcell_of(const Params &P, uint4 q) {
 }
 
 // ------------------------------------------------------- shared memory
-template <typename Real, int G>
+// A group's scratch for step items.  S, P and the pair tables describe the
+// group's system and stay from item to item (they do not change during a
+// launch): read from shared memory, a step's first accesses do not go to the
+// L2 cache, which they would after every grid barrier (its fence invalidates
+// the L1 cache).  The other arrays hold the item's beads; a group whose item
+// stays the same from step to step (KEEP: the persistent kernel's overlapped
+// mode) finds them there at the next step, and has room for what else it can
+// keep.  The other modes do without: shared memory taken here is L1 cache
+// lost to the position gathers, which they miss more.
+//
+// Pair tables: the Lennard-Jones factors as 8-byte entries and the charge
+// products apart, which only beads of a charged type (qrow) load: the step is
+// bound by the wavefronts of its shared and global loads, and a 16-byte entry
+// took at least four of them per warp where these take two or three.
+template <int NB>
+struct ItemKeep {
+    uint4 spos[NB];
+    int4 first[NL_BLOCK];                     // each thread's rows 0 .. 3
+    int cnt[NL_BLOCK];                        // each thread's column length
+    int sslot[NB][NL_PART];                   // list indices of the bonded partners
+};
+struct ItemKeepNone {};
+
+template <typename Real, int G, bool KEEP>
 struct StepSmem {
     using V4 = typename Vec4<Real>::T;
+    struct __align__(2 * sizeof(Real)) LJ { Real f12, f6; };
     static constexpr int NB = NL_BLOCK / G;   // beads of a step item
-    V4 tab[256];                              // 12 C12, 6 C6, qq per type pair
+    uint4 spart[NB][NL_PART];
     V4 svel[NB];
     uint4 sxref[NB];
-    uint4 spart[NB][NL_PART];
+    LJ tab[256];                              // 12 C12, 6 C6 per type pair
+    Real tabq[256];                           // f qi qj / eps_r
     Real kered[2][NB];
+    int sid[NB];
     int sviol;
     int redo;
+    unsigned qrow;                            // bit i: type i has a charge product that is not zero
+    SysDev S;
+    ParamsHot P;
+    typename std::conditional<KEEP, ItemKeep<NB>, ItemKeepNone>::type keep;
 };
 
 // What a step item of the persistent kernel waits for when the previous
@@ -110,12 +141,12 @@ __device__ __forceinline__ unsigned ld_relaxed32(const unsigned *p) {
 // The thermostat factor of coupling group grp for a step beside the close.
 // FP32: the factor and its close sequence share one 64-bit word (one relaxed
 // load gives both, no fence); FP64: the sequence, a fence, then the factor.
+// w: the word as loaded earlier in the step (FP32).
 template <typename Real>
-__device__ Real alpha_beside_close(Counters &C, int grp, const PipeWait &pw) {
+__device__ Real alpha_beside_close(Counters &C, int grp, const PipeWait &pw, unsigned long long w) {
     constexpr long long LIMIT = 1ll << 24;
     if (sizeof(Real) == 4) {
         const unsigned want = (unsigned)pw.close_target;
-        unsigned long long w = ld_relaxed64(&C.alpha_pack[grp]);
         for (long long it = 0; (unsigned)(w >> 32) != want; ++it) {
             if (it > LIMIT) { atomicOr(&C.err, ERR_TIMEOUT); break; }
             w = ld_relaxed64(&C.alpha_pack[grp]);
@@ -131,7 +162,7 @@ __device__ Real alpha_beside_close(Counters &C, int grp, const PipeWait &pw) {
 // Thread 0 of a step item after a trial: wait (bounded) for the trial's
 // marks; true when the trial exchanged bead types this item sees, so its
 // forces must be summed again.
-static __device__ bool pipe_wait(const SysDev &S, const PipeWait &pw, int item) {
+static __device__ bool pipe_wait(const SysDev &S, int mark_words, const PipeWait &pw, int item) {
     Counters &C = *S.c;
     constexpr long long LIMIT = 1ll << 24;
     bool ok = true, redo = false;
@@ -139,7 +170,7 @@ static __device__ bool pipe_wait(const SysDev &S, const PipeWait &pw, int item) 
         if (it > LIMIT) { ok = false; break; }
     asm volatile("fence.acq_rel.gpu;" ::: "memory");
     if (ok) {
-        const unsigned w = __ldcg(&S.tmark[(size_t)(pw.T & 1) * S.p->mark_words + item / 32]);
+        const unsigned w = __ldcg(&S.tmark[(size_t)(pw.T & 1) * mark_words + item / 32]);
         if ((w >> (item & 31)) & 1u) {
             for (long long it = 0; ld_relaxed64(&C.trial) <= pw.T; ++it)
                 if (it > LIMIT) { ok = false; break; }
@@ -167,9 +198,9 @@ struct BuildSmem {
 
 constexpr size_t cmax(size_t a, size_t b) { return a > b ? a : b; }
 
-template <typename Real, int G>
+template <typename Real, int G, bool KEEP>
 constexpr size_t group_smem() {
-    return (cmax(cmax(sizeof(StepSmem<Real, G>), sizeof(BuildSmem)), sizeof(TrialSmem)) + 15) & ~(size_t)15;
+    return (cmax(cmax(sizeof(StepSmem<Real, G, KEEP>), sizeof(BuildSmem)), sizeof(TrialSmem)) + 15) & ~(size_t)15;
 }
 
 // ------------------------------------------------------------ build items
@@ -201,14 +232,15 @@ __device__ __forceinline__ int loct_of(const Params &P, uint4 q) {
 // position buffer par, ranked within their cell by (octant, id): beads next to
 // each other in the list are close in space.  The first list index of a cell
 // is the number of beads in the cells before it, summed here by the whole
-// group (every item sums its own prefix: no serial scan).
-static __device__ void nl_place_item(const SysDev &S, int c0, int par, const Grp &g, BuildSmem &sm) {
+// group (every item sums its own prefix: no serial scan).  run: the beads of a
+// list-build task at most.
+static __device__ void nl_place_item(const SysDev &S, int c0, int par, int run, const Grp &g, BuildSmem &sm) {
     const Params &P = *S.p;
     int part = 0, tpart = 0;
     for (int q = g.t; q < c0; q += GRP) {
         const int m = min(__ldcg(&S.lcell_count[q]), P.lcapc);
         part += m;
-        tpart += nl_build_tasks(m);
+        tpart += nl_build_tasks(m, run);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -223,7 +255,7 @@ static __device__ void nl_place_item(const SysDev &S, int c0, int par, const Grp
     for (int q = c0; q < c; ++q) {
         const int m = min(__ldcg(&S.lcell_count[q]), P.lcapc);
         first += m;
-        tfirst += nl_build_tasks(m);
+        tfirst += nl_build_tasks(m, run);
     }
     g.sync();
     if (c >= P.n_lcells) return;
@@ -232,7 +264,7 @@ static __device__ void nl_place_item(const SysDev &S, int c0, int par, const Grp
     if (lane == 0) S.lcell[c] = lc;
     // the cell's list-build tasks (cell, tasks << 16 | task) and, after the
     // last cell, the number of tasks
-    const int ntk = nl_build_tasks(cnt);
+    const int ntk = nl_build_tasks(cnt, run);
     for (int x = lane; x < ntk; x += 32) S.btask[tfirst + x] = make_int2(c, (ntk << 16) | x);
     if (lane == 0 && c == P.n_lcells - 1) S.c->nbtask = tfirst + ntk;
     uint4 *cur = S.lpos + (size_t)par * P.n;
@@ -261,26 +293,25 @@ static __device__ void nl_place_item(const SysDev &S, int c0, int par, const Grp
     }
 }
 
-// One list-build task: the lists of beads b0 .. b0 + nb - 1 (at most
-// NLB_BEADS, a run of one list-build cell's beads) for one warp.  The 27
-// neighbour cells are read in a frame centred on the cell (exact integer
-// offsets as floats; with 3 or more cells per edge every partner within rl of
-// a bead of the cell has an offset below half a box, so the frame difference
-// is the minimum image), cell by cell, 32 candidates at a time; those near
-// the box around the task's beads go to a ring in shared memory, and every 32
-// of them lane u tests candidate u against every bead of the task: a ballot
-// per bead gives the partners their list entries in candidate order (cells
-// in order, beads in list order within a cell), dealt to the columns in turn.
+// One list-build task: the lists of beads b0 .. b0 + nb - 1 (at most NB, a run
+// of one list-build cell's beads) for one warp.  The 27 neighbour cells are
+// read in a frame centred on the cell (exact integer offsets as floats; with 3
+// or more cells per edge every partner within rl of a bead of the cell has an
+// offset below half a box, so the frame difference is the minimum image), 32
+// candidates at a time (cells in order, beads in list order within a cell);
+// those near the box around the task's beads go to a ring in shared memory,
+// and every 32 of them lane u tests candidate u against every bead of the
+// task: a ballot per bead gives the partners their list entries in candidate
+// order, dealt to the columns in turn.
 //
-// PF: the positions of the next two chunks of candidates are loaded while
-// the current one is filtered (shorter latency per task, more registers:
-// taken where a build is one round of tasks on an otherwise idle GPU, the
-// persistent kernel of lone systems and the separate launches; a batch's
-// partitioned kernel, bound by its instruction issue, walks without).
-template <int G, bool PF>
+// A lane per candidate and a vote per bead measured faster here than a lane
+// per bead with masks of partners (fewer tests, but 30% of a cell's lanes
+// idle, two passes for a cell of more than 32 beads and entries written lane
+// by lane): 51 against 63 us for the 1152-lipid bilayer's build.
+template <int G, int NB>
 __device__ void nl_build_task(const SysDev &S, int task, int par, int lane, BuildWarp &sw) {
-    constexpr int NL_G = G;
     constexpr unsigned FULL = 0xffffffffu;
+    static_assert(NB <= NLB_BEADS, "scratch for NLB_BEADS beads");
     const Params &P = *S.p;
     Counters &C = *S.c;
     const int2 tk = S.btask[task];
@@ -288,7 +319,8 @@ __device__ void nl_build_task(const SysDev &S, int task, int par, int lane, Buil
     const uint4 *cur = S.lpos + (size_t)par * P.n;
     const int nx = P.ln[0], ny = P.ln[1], nz = P.ln[2];
     const int cz = c / (nx * ny), cxy = c - cz * nx * ny, cy = cxy / nx, cx = cxy - cy * nx;
-    // lane q < 27: first list index and bead count of neighbour cell q (13: the cell itself)
+    // lane q < 27: first list index and bead count of neighbour cell q (13:
+    // the cell itself), and the number of candidates in the cells before it
     int2 nbq = make_int2(0, 0);
     if (lane < 27) {
         const int dz = lane / 9 - 1, dy = (lane / 3) % 3 - 1, dx = lane % 3 - 1;
@@ -298,7 +330,16 @@ __device__ void nl_build_task(const SysDev &S, int task, int par, int lane, Buil
         z += z < 0 ? nz : (z >= nz ? -nz : 0);
         nbq = S.lcell[(z * ny + y) * nx + x];
     }
+    int off = nbq.y;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int x = __shfl_up_sync(FULL, off, d);
+        if (lane >= d) off += x;
+    }
+    const int M = __shfl_sync(FULL, off, 31);
+    off -= nbq.y;                                     // lanes 27 .. 31: M
     const int i0 = __shfl_sync(FULL, nbq.x, 13), ni = __shfl_sync(FULL, nbq.y, 13);
+    const int first_of = nbq.x - off;                 // list index of candidate t of cell q: t + first_of
     if (sub == 0 && lane == 0) S.lcell_count[c] = 0;   // counted afresh at the next build
     // this task's run of the cell's beads (the runs differ by one bead at most)
     const int b0 = sub * ni / ntk, nbw = (sub + 1) * ni / ntk - b0, kb = i0 + b0;
@@ -307,39 +348,58 @@ __device__ void nl_build_task(const SysDev &S, int task, int par, int lane, Buil
     const uint32_t oz = (uint32_t)(((unsigned long long)(2 * cz + 1) * P.lcwu[2]) >> 1);
     const float q0 = P.qsf[0], q1 = P.qsf[1], q2 = P.qsf[2];
     const float rl2 = P.rl2f;
-    const int capg = P.lcap / NL_G;
     const unsigned ltmask = (1u << lane) - 1u;
+    // candidate t: cell q with off[q] <= t < off[q + 1] (a cell with no beads
+    // has its successor's offset: the last q that qualifies)
+    auto load = [&](int t, uint4 &p, int &k) {
+        int q = 0;
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) {
+            const int o = __shfl_sync(FULL, off, q + d);
+            if (o <= t) q += d;
+        }
+        k = __shfl_sync(FULL, first_of, q) + t;
+        p = t < M ? cur[k] : make_uint4(0u, 0u, 0u, 0u);
+    };
+    uint4 p1;
+    int k1;
+    load(lane, p1, k1);
     // lane b holds bead b of the run (its frame position and exclusions also
     // in shared memory, where every lane reads them)
     const bool act = lane < nbw;
     const int ki = kb + (act ? lane : 0);
     const uint4 pi = cur[ki];
-    const float xi = (float)(int)(pi.x - ox) * q0, yi = (float)(int)(pi.y - oy) * q1,
-                zi = (float)(int)(pi.z - oz) * q2;
     const uint32_t lip = pi.w >> 12;
     const uint32_t em = lip ? P.excl[meta_k(pi.w)] : 0u;
-    if (act) {
-        sw.sb[lane] = make_float4(xi, yi, zi, __uint_as_float(pi.w >> 8));   // (lipid + 1) << 4 | k
-        sw.sbe[lane] = em;
-    }
-    // the box around the run's beads
-    float lo0 = act ? xi : 3e30f, lo1 = act ? yi : 3e30f, lo2 = act ? zi : 3e30f;
-    float hi0 = act ? xi : -3e30f, hi1 = act ? yi : -3e30f, hi2 = act ? zi : -3e30f;
+    const bool lipids = __any_sync(FULL, act && em != 0u);
+    float lo0, lo1, lo2, hi0, hi1, hi2;               // the box around the run's beads
+    {
+        const float xi = (float)(int)(pi.x - ox) * q0, yi = (float)(int)(pi.y - oy) * q1,
+                    zi = (float)(int)(pi.z - oz) * q2;
+        if (act) {
+            sw.sb[lane] = make_float4(xi, yi, zi, __uint_as_float(pi.w >> 8));   // (lipid + 1) << 4 | k
+            sw.sbe[lane] = em;
+        }
+        lo0 = act ? xi : 3e30f; lo1 = act ? yi : 3e30f; lo2 = act ? zi : 3e30f;
+        hi0 = act ? xi : -3e30f; hi1 = act ? yi : -3e30f; hi2 = act ? zi : -3e30f;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        lo0 = fminf(lo0, __shfl_xor_sync(FULL, lo0, o));
-        lo1 = fminf(lo1, __shfl_xor_sync(FULL, lo1, o));
-        lo2 = fminf(lo2, __shfl_xor_sync(FULL, lo2, o));
-        hi0 = fmaxf(hi0, __shfl_xor_sync(FULL, hi0, o));
-        hi1 = fmaxf(hi1, __shfl_xor_sync(FULL, hi1, o));
-        hi2 = fmaxf(hi2, __shfl_xor_sync(FULL, hi2, o));
+        for (int o = NB / 2; o > 0; o >>= 1) {        // the beads are in the first NB lanes
+            lo0 = fminf(lo0, __shfl_xor_sync(FULL, lo0, o));
+            lo1 = fminf(lo1, __shfl_xor_sync(FULL, lo1, o));
+            lo2 = fminf(lo2, __shfl_xor_sync(FULL, lo2, o));
+            hi0 = fmaxf(hi0, __shfl_xor_sync(FULL, hi0, o));
+            hi1 = fmaxf(hi1, __shfl_xor_sync(FULL, hi1, o));
+            hi2 = fmaxf(hi2, __shfl_xor_sync(FULL, hi2, o));
+        }
+        lo0 = __shfl_sync(FULL, lo0, 0); lo1 = __shfl_sync(FULL, lo1, 0); lo2 = __shfl_sync(FULL, lo2, 0);
+        hi0 = __shfl_sync(FULL, hi0, 0); hi1 = __shfl_sync(FULL, hi1, 0); hi2 = __shfl_sync(FULL, hi2, 0);
     }
     __syncwarp();
     // loop invariants in registers (stores through the list pointer could
     // otherwise alias them and force reloads from global memory)
-    int *const nl = S.nl;
-    const size_t lrow = (size_t)P.npad * G;
-    const unsigned lcapg = (unsigned)(capg * NL_G);   // entries a bead's list holds
+    int *const nl = S.nl + (size_t)kb * (4 * G);
+    const size_t lblk = nl_block_stride<G>(P.npad);
+    const unsigned cap = (unsigned)(P.lcap / G * G);  // entries a bead's list holds
     int base = 0;                                     // lane b: entries of bead b so far
     unsigned head = 0, tail = 0;                      // ring entries head .. tail - 1 wait for their tests
     // lane u tests ring entry head + u (u < nt) against every bead of the run
@@ -350,26 +410,28 @@ __device__ void nl_build_task(const SysDev &S, int task, int par, int lane, Buil
         const int sl = (int)((head + (unsigned)lane) & 63u);
         const float4 e = sw.nf[sl];
         const int kj = sw.nk[sl];
-        const uint32_t jkey = __float_as_uint(e.w) >> 8;   // (lipid + 1) << 4 | k
-        const uint32_t jk = jkey & 15u;
-        unsigned bal[NLB_BEADS];
+        unsigned bal[NB];
 #pragma unroll
-        for (int b = 0; b < NLB_BEADS; ++b) {
+        for (int b = 0; b < NB; ++b) {
             const float4 bi = sw.sb[b];
             const float dx = bi.x - e.x, dy = bi.y - e.y, dz = bi.z - e.z;
             const float r2 = dx * dx + dy * dy + dz * dz;
+            bal[b] = __ballot_sync(FULL, b < nbw && have && r2 < rl2 && kj != kb + b);
+        }
+        if (lipids) {
             // excluded: the same lipid ((lipid + 1) equal) and a bonded local index
-            const bool excl = (__float_as_uint(bi.w) ^ jkey) < 16u && ((sw.sbe[b] >> jk) & 1u);
-            const bool in = b < nbw && have && r2 < rl2 && !excl && kj != kb + b;
-            bal[b] = __ballot_sync(FULL, in);
+            const uint32_t jkey = __float_as_uint(e.w) >> 8, jk = jkey & 15u;   // (lipid + 1) << 4 | k
+#pragma unroll
+            for (int b = 0; b < NB; ++b)
+                bal[b] &= ~__ballot_sync(FULL, (__float_as_uint(sw.sb[b].w) ^ jkey) < 16u && ((sw.sbe[b] >> jk) & 1u));
         }
 #pragma unroll
-        for (int b = 0; b < NLB_BEADS; ++b) {
+        for (int b = 0; b < NB; ++b) {
             if (bal[b]) {
                 const int bb = __shfl_sync(FULL, base, b);
                 if ((bal[b] >> lane) & 1u) {
                     const unsigned ei = (unsigned)bb + __popc(bal[b] & ltmask);
-                    if (ei < lcapg) nl[(size_t)(kb + b) * NL_G + (size_t)(ei / NL_G) * lrow + ei % NL_G] = kj;
+                    if (ei < cap) nl[(size_t)(ei / (4 * G)) * lblk + b * (4 * G) + ei % G * 4 + ei / G % 4] = kj;
                 }
                 if (lane == b) base = bb + __popc(bal[b]);
             }
@@ -377,66 +439,23 @@ __device__ void nl_build_task(const SysDev &S, int task, int par, int lane, Buil
         head += (unsigned)nt;
         __syncwarp();                                 // the tested slots may be written next
     };
-    // the candidates cell by cell, 32 at a time (a chunk: j0 .. j0 + 31 of
-    // cell q)
-    int q = 0, j0 = -32, qf = __shfl_sync(FULL, nbq.x, 0), qn = __shfl_sync(FULL, nbq.y, 0);
-    auto next_chunk = [&]() {
-        j0 += 32;
-        while (j0 >= qn && q < 27) {
-            ++q;
-            j0 = 0;
-            qf = __shfl_sync(FULL, nbq.x, q);      // lanes 27 .. 31 hold no cell: q = 27 ends the walk
-            qn = __shfl_sync(FULL, nbq.y, q);
-        }
-    };
-    auto load = [&](uint4 &p, int &k, bool &v) {
-        const int j = j0 + lane;
-        v = q < 27 && j < qn;
-        k = qf + j;
-        p = v ? cur[k] : make_uint4(0u, 0u, 0u, 0u);
-    };
-    uint4 p1 = make_uint4(0u, 0u, 0u, 0u), p2 = p1;
-    int k1 = 0, k2 = 0;
-    bool v1 = false, v2 = false, m2 = false;
-    next_chunk();
-    bool m1 = q < 27;                                 // a chunk is left
-    if (PF) {
-        load(p1, k1, v1);
-        next_chunk();
-        m2 = q < 27;
-        load(p2, k2, v2);
-    }
-    while (m1) {
-        uint4 pj;
-        int kj;
-        bool v;
-        if (PF) {
-            pj = p1; kj = k1; v = v1;
-            p1 = p2; k1 = k2; v1 = v2; m1 = m2;
-            next_chunk();
-            m2 = q < 27;
-            load(p2, k2, v2);
-        } else {
-            load(pj, kj, v);
-            next_chunk();
-            m1 = q < 27;
-        }
-        bool near = false;
-        float4 e = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (v) {
-            e = make_float4((float)(int)(pj.x - ox) * q0, (float)(int)(pj.y - oy) * q1,
-                            (float)(int)(pj.z - oz) * q2, __uint_as_float(pj.w));
-            // the candidate is within rl of the box around the run's beads
-            const float gx = fmaxf(fmaxf(lo0 - e.x, e.x - hi0), 0.f);
-            const float gy = fmaxf(fmaxf(lo1 - e.y, e.y - hi1), 0.f);
-            const float gz = fmaxf(fmaxf(lo2 - e.z, e.z - hi2), 0.f);
-            near = gx * gx + gy * gy + gz * gz < rl2;
-        }
+    for (int tb = 0; tb < M; tb += 32) {
+        const uint4 p = p1;
+        const int k = k1;
+        const bool v = tb + lane < M;
+        if (tb + 32 < M) load(tb + 32 + lane, p1, k1);   // in flight while this chunk is filtered and tested
+        const float ax = (float)(int)(p.x - ox) * q0, ay = (float)(int)(p.y - oy) * q1,
+                    az = (float)(int)(p.z - oz) * q2;
+        // the candidate is within rl of the box around the run's beads
+        const float gx = fmaxf(fmaxf(lo0 - ax, ax - hi0), 0.f);
+        const float gy = fmaxf(fmaxf(lo1 - ay, ay - hi1), 0.f);
+        const float gz = fmaxf(fmaxf(lo2 - az, az - hi2), 0.f);
+        const bool near = v && gx * gx + gy * gy + gz * gz < rl2;
         const unsigned bn = __ballot_sync(FULL, near);
         if (near) {
             const int sl = (int)((tail + (unsigned)__popc(bn & ltmask)) & 63u);
-            sw.nf[sl] = e;
-            sw.nk[sl] = kj;
+            sw.nf[sl] = make_float4(ax, ay, az, __uint_as_float(p.w));
+            sw.nk[sl] = k;
         }
         tail += (unsigned)__popc(bn);
         __syncwarp();
@@ -444,9 +463,11 @@ __device__ void nl_build_task(const SysDev &S, int task, int par, int lane, Buil
     }
     if (tail != head) test((int)(tail - head));
     if (act) {
-        for (int col = 0; col < NL_G; ++col) {
-            const int cnt = base > col ? (base - col + NL_G - 1) / NL_G : 0;
-            S.nl_n[(size_t)ki * NL_G + col] = min(cnt, capg);
+        for (int col = 0; col < G; ++col) {
+            const int cnt = min(base > col ? (base - col + G - 1) / G : 0, (int)cap / G);
+            S.nl_n[(size_t)ki * G + col] = cnt;
+            // the last group of 4 rows filled up with the bead itself (the step walks whole groups)
+            for (int r = cnt; r & 3; ++r) S.nl[nl_at<G>(P.npad, ki, r, col)] = ki;
         }
         if (base > P.lcap) atomicOr(&C.err, ERR_CELL_OVERFLOW);
         if (lip != 0) {
@@ -461,7 +482,7 @@ __device__ void nl_build_task(const SysDev &S, int task, int par, int lane, Buil
 // The list-build tasks of the systems whose flag is set, dealt to warps
 // gw = 0 .. nw - 1 in turn: task x of the batch (the systems' tasks one after
 // another) goes to warp x mod nw.  Every lane of a warp calls it alike.
-template <int G, typename Flag, typename Par>
+template <int G, int NB, typename Flag, typename Par>
 __device__ void nl_build_dealt(const SysDev *sys, int n_sys, int gw, int nw, int lane, BuildWarp &sw, Flag flag,
                                Par par) {
     constexpr unsigned FULL = 0xffffffffu;
@@ -483,80 +504,128 @@ __device__ void nl_build_dealt(const SysDev *sys, int n_sys, int gw, int nw, int
             int t = gw - (int)(((long long)off + ej) % nw);
             if (t < 0) t += nw;
             const SysDev &S = sys[q0 + j];
-            for (; t < Tj; t += nw) nl_build_task<G, true>(S, t, par(S), lane, sw);
+            for (; t < Tj; t += nw) nl_build_task<G, NB>(S, t, par(S), lane, sw);
         }
         off = (int)(((long long)off + __shfl_sync(FULL, incl, 31)) % nw);
     }
 }
 
-// A list entry: read once per step, so it skips L1 (which keeps the
+// Four list entries: read once per step, so they skip L1 (which keeps the
 // positions and tables the step reuses)
-__device__ __forceinline__ int ld_list(const int *p) {
-    int v;
-    asm volatile("ld.global.nc.L1::no_allocate.b32 %0, [%1];" : "=r"(v) : "l"(p));
+__device__ __forceinline__ int4 ld_list(const int4 *p) {
+    int4 v;
+    asm volatile("ld.global.nc.L1::no_allocate.v4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
     return v;
 }
 
 // ------------------------------------------------------------- step item
+// Copies of a group's system into its scratch: pointers, scalars and
+// topology, pair tables (the caller's group barrier follows).
+template <typename Real, int G, bool KEEP>
+__device__ void load_system(const SysDev &Sg, const Grp &g, StepSmem<Real, G, KEEP> &sm) {
+    static_assert(sizeof(SysDev) % 4 == 0 && sizeof(ParamsHot) % 4 == 0, "copied by words");
+    const Params &Pg = *Sg.p;
+    for (int x = g.t; x < (int)(sizeof(SysDev) / 4); x += GRP)
+        reinterpret_cast<int *>(&sm.S)[x] = reinterpret_cast<const int *>(&Sg)[x];
+    for (int x = g.t; x < (int)(sizeof(ParamsHot) / 4); x += GRP)
+        reinterpret_cast<int *>(&sm.P)[x] = reinterpret_cast<const int *>(static_cast<const ParamsHot *>(&Pg))[x];
+    constexpr bool F32 = sizeof(Real) == 4;
+    unsigned qrow = 0;
+    for (int x = g.t; x < 256; x += GRP) {
+        sm.tab[x].f12 = F32 ? (Real)Pg.f12f[x] : (Real)(12.0 * Pg.c12[x]);
+        sm.tab[x].f6 = F32 ? (Real)Pg.f6f[x] : (Real)(6.0 * Pg.c6[x]);
+        const Real q = F32 ? (Real)Pg.qqf[x] : (Real)Pg.qq[x];
+        sm.tabq[x] = q;
+        if (q != (Real)0) qrow |= 1u << (x >> 4);
+    }
+    if (g.t == 0) {
+        sm.sviol = 0;                          // afterwards cleared by every item's end
+        sm.qrow = 0;
+    }
+    g.sync();
+    if (qrow) atomicOr(&sm.qrow, qrow);
+}
+
 // One MD step of the beads k0 .. k0 + NL_BEADS - 1 (list order): positions
 // read from buffer par, written to buffer par ^ 1 and to the id-ordered
 // array.  The item's kinetic energy goes to an integer slot; a bead that
-// moved farther than the list allows sets *viol.
-template <typename Real, int LAM, int G>
-__device__ void nl_step_item(const SysDev &S, int k0, int par, int *viol, const Grp &g, StepSmem<Real, G> &sm,
-                             bool load_tables = true, const PipeWait *pw = nullptr) {
+// moved farther than the list allows sets *viol.  The group's system is in
+// sm (load_system).  kept: sm also holds this same item's beads from the step
+// before, with no list build in between.
+template <typename Real, int LAM, int G, bool KEEP>
+__device__ __forceinline__ void nl_step_item(int k0, int par, int *viol, const Grp &g, StepSmem<Real, G, KEEP> &sm,
+                                             const PipeWait *pw = nullptr, bool kept = false) {
     constexpr int NL_G = G, NL_BEADS = NL_BLOCK / G;
     using V4 = typename Vec4<Real>::T;
     constexpr bool F32 = sizeof(Real) == 4;
-    const Params &P = *S.p;
+    const SysDev &S = sm.S;
+    const ParamsHot &P = sm.P;
     Counters &C = *S.c;
     const int t = g.t, il = t / NL_G, gl = t % NL_G;
     const int n = P.n;
     const int k = k0 + il;
     const bool valid = k < n;
     const uint4 *__restrict__ cur = S.lpos + (size_t)par * n;
-    uint4 *nxt = S.lpos + (size_t)(par ^ 1) * n;
+    const int4 *__restrict__ lst = reinterpret_cast<const int4 *>(S.nl) + (size_t)k * NL_G + gl;
+    const size_t rs = (size_t)P.npad * G;      // from one group of 4 rows to the next
+    auto rows4 = [&](const int4 *p) {
+        const int4 v = ld_list(p);
+        return make_int4(MDAS_IDX(C, v.x, n), MDAS_IDX(C, v.y, n), MDAS_IDX(C, v.z, n), MDAS_IDX(C, v.w, n));
+    };
     // this lane's list column: its first rows are loaded before anything else
     // (rows 0 .. 3 always exist; entries past the end hold valid indices)
-    const int *__restrict__ lst = S.nl + (size_t)k * NL_G + gl;
-    const size_t rs = (size_t)P.npad * G;
-    int j0 = MDAS_IDX(C, ld_list(lst), n), j1 = MDAS_IDX(C, ld_list(lst + rs), n);
-    int j2 = MDAS_IDX(C, ld_list(lst + 2 * rs), n), j3 = MDAS_IDX(C, ld_list(lst + 3 * rs), n);
+    int4 j;
+    int cnt = 0;
     uint4 pi = make_uint4(0u, 0u, 0u, 0u);
-    int cnt = 0, id = 0;
-    if (valid) {
-        pi = cur[k];
-        cnt = S.nl_n[(size_t)k * NL_G + gl];
-    }
-    if (load_tables) {                         // else still there from the group's previous item
-        for (int x = t; x < 256; x += GRP) {
-            V4 e;
-            if (F32) {
-                e.x = (Real)P.f12f[x]; e.y = (Real)P.f6f[x]; e.z = (Real)P.qqf[x];
-            } else {
-                e.x = (Real)(12.0 * P.c12[x]); e.y = (Real)(6.0 * P.c6[x]); e.z = (Real)P.qq[x];
-            }
-            e.w = (Real)0;
-            sm.tab[x] = e;
+    bool loaded = false;
+    if constexpr (KEEP) {
+        if (kept) {
+            j = sm.keep.first[t];
+            if (valid) pi = sm.keep.spos[il];
+            cnt = sm.keep.cnt[t];
+            loaded = true;
         }
-        if (t == 0) sm.sviol = 0;              // afterwards cleared by every item's end
-        g.sync();
+    }
+    if (!loaded) {
+        j = rows4(lst);
+        if (valid) {
+            pi = cur[k];
+            cnt = S.nl_n[(size_t)k * NL_G + gl];
+        }
+        if constexpr (KEEP) {
+            sm.keep.first[t] = j;
+            sm.keep.cnt[t] = cnt;
+        }
     }
     // the first row group's positions, then (while they arrive) the copies
-    // into shared memory the update needs: velocity and build position by
-    // lanes 0 and 1, the bonded partners spread over the bead's lanes
-    uint4 q0 = cur[j0], q1 = cur[j1], q2 = cur[j2], q3 = cur[j3];
+    // into shared memory the update needs: the bonded partners' positions
+    // spread over the bead's lanes, and what a group does not hold yet:
+    // velocity, build position, id, partner slots
+    uint4 q0 = cur[j.x], q1 = cur[j.y], q2 = cur[j.z], q3 = cur[j.w];
     if (valid) {
-        if (gl == 0) {
-            id = MDAS_IDX(C, S.lid[k], n);
-            const char *gv = reinterpret_cast<const char *>(reinterpret_cast<const V4 *>(S.vel) + id);
-            for (int h = 0; h < (int)sizeof(V4); h += 16) cp_async16(reinterpret_cast<char *>(&sm.svel[il]) + h, gv + h);
+        if (!loaded) {
+            if (gl == 0) {
+                const int id = MDAS_IDX(C, S.lid[k], n);
+                sm.sid[il] = id;
+                const char *gv = reinterpret_cast<const char *>(reinterpret_cast<const V4 *>(S.vel) + id);
+                for (int h = 0; h < (int)sizeof(V4); h += 16)
+                    cp_async16(reinterpret_cast<char *>(&sm.svel[il]) + h, gv + h);
+            }
+            if (gl == 1 % NL_G) cp_async16(&sm.sxref[il], S.xref + k);
         }
-        if (gl == 1 % NL_G) cp_async16(&sm.sxref[il], S.xref + k);
         if (meta_lip(pi.w) >= 0) {
-            const int kl = meta_k(pi.w);
-            for (int p = gl; p < P.npart[kl]; p += NL_G)
-                cp_async16(&sm.spart[il][p], cur + MDAS_IDX(C, S.bslot[(size_t)k * NL_PART + p], n));
+            const int np = P.npart[meta_k(pi.w)];
+            for (int p = gl; p < np; p += NL_G) {
+                int slot;
+                if constexpr (KEEP) {                  // a lane reads back the slots it wrote itself
+                    if (!loaded) sm.keep.sslot[il][p] = MDAS_IDX(C, S.bslot[(size_t)k * NL_PART + p], n);
+                    slot = sm.keep.sslot[il][p];
+                } else {
+                    slot = MDAS_IDX(C, S.bslot[(size_t)k * NL_PART + p], n);
+                }
+                cp_async16(&sm.spart[il][p], cur + slot);
+            }
         }
         asm volatile("cp.async.commit_group;\n" ::: "memory");
     }
@@ -572,52 +641,68 @@ __device__ void nl_step_item(const SysDev &S, int k0, int par, int *viol, const 
     const Real dsc = LAM == 2 ? (F32 ? (Real)P.sc_deltaf : (Real)P.sc_delta) : (Real)0;
     const float qs0 = P.qsf[0], qs1 = P.qsf[1], qs2 = P.qsf[2];
     int tai = meta_ta(pi.w) * 16, tbi = meta_tb(pi.w) * 16;
+    const unsigned qrow = sm.qrow;
+    bool charged = ((qrow >> meta_ta(pi.w)) | (ALCH ? qrow >> meta_tb(pi.w) : 0u)) & 1u;
     Real ax = 0, ay = 0, az = 0;
     Real wx = 0, wy = 0, wz = 0;               // PC: sums of f d_a^2 over this lane's entries
 
-    auto pair = [&](uint4 pj, bool ok) {
+    // A pair in two halves.  cull: the separation (one rounding of the exact
+    // integer offsets), r^2, whether the pair is inside the cutoff and, in
+    // FP32, whether r^2 lies within float rounding of it (decided from the
+    // exact offsets by in_exact; about one entry in 2 * 10^4).  A partner at
+    // zero distance (a padding entry is the bead itself) is outside.
+    struct Sep { Real x, y, z, r2; uint32_t w; bool in, edge; };
+    auto cull = [&](uint4 pj) {
+        Sep e;
         const int ix = (int)(pi.x - pj.x), iy = (int)(pi.y - pj.y), iz = (int)(pi.z - pj.z);
-        Real dx, dy, dz;
         if (F32) {
-            dx = (Real)((float)ix * qs0);
-            dy = (Real)((float)iy * qs1);
-            dz = (Real)((float)iz * qs2);
+            e.x = (Real)((float)ix * qs0);
+            e.y = (Real)((float)iy * qs1);
+            e.z = (Real)((float)iz * qs2);
         } else {
-            dx = (Real)((double)ix * P.qs[0]);
-            dy = (Real)((double)iy * P.qs[1]);
-            dz = (Real)((double)iz * P.qs[2]);
+            e.x = (Real)((double)ix * P.qs[0]);
+            e.y = (Real)((double)iy * P.qs[1]);
+            e.z = (Real)((double)iz * P.qs[2]);
         }
-        const Real r2 = fmr(dx, dx, fmr(dy, dy, dz * dz));
-        bool in = ok & (r2 < rc2) & (r2 > (Real)0);
-        if (F32 && in && r2 >= rc2lo) {
-            // within float rounding of the cutoff: decide from the exact offsets
-            const double ex = (double)ix * P.qs[0], ey = (double)iy * P.qs[1], ez = (double)iz * P.qs[2];
-            in = ex * ex + ey * ey + ez * ez < P.rc2;
-        }
-        const Real r2c = in ? r2 : (Real)1;        // out of range: computed, then dropped
-        const uint32_t mj = pj.w;
-        const V4 ca = sm.tab[tai + meta_ta(mj)];
-        Real f12 = ca.x, f6 = ca.y, qq = ca.z;
-        V4 cb = ca;
+        e.r2 = fmr(e.x, e.x, fmr(e.y, e.y, e.z * e.z));
+        e.w = pj.w;
+        e.in = (e.r2 < rc2lo) & (e.r2 > (Real)0);
+        e.edge = F32 && (e.r2 < rc2) & !(e.r2 < rc2lo);
+        return e;
+    };
+    auto in_exact = [&](uint4 pj) {
+        const double ex = (double)(int)(pi.x - pj.x) * P.qs[0], ey = (double)(int)(pi.y - pj.y) * P.qs[1],
+                     ez = (double)(int)(pi.z - pj.z) * P.qs[2];
+        return ex * ex + ey * ey + ez * ez < P.rc2;
+    };
+    // add: the force (a pair outside is computed and dropped: no branch, so
+    // the halves of a row group interleave)
+    auto add = [&](const Sep &e) {
+        const uint32_t mj = e.w;
+        const auto ca = sm.tab[tai + meta_ta(mj)];
+        Real f12 = ca.f12, f6 = ca.f6, qq = (Real)0;
+        if (charged) qq = sm.tabq[tai + meta_ta(mj)];
+        auto cb = ca;
         if (ALCH) {
             cb = sm.tab[tbi + meta_tb(mj)];
-            f12 = fmr((Real)1 - lam, f12, lam * cb.x);
-            f6 = fmr((Real)1 - lam, f6, lam * cb.y);
-            qq = fmr((Real)1 - lam, qq, lam * cb.z);
+            f12 = fmr((Real)1 - lam, f12, lam * cb.f12);
+            f6 = fmr((Real)1 - lam, f6, lam * cb.f6);
+            if (charged) qq = fmr((Real)1 - lam, qq, lam * sm.tabq[tbi + meta_tb(mj)]);
         }
         Real rinv, r2inv, r6inv;
         if (F32) {
             // 1/r^2: hardware estimate and one Newton-Raphson step
-            float r2i;
-            asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r2i) : "f"((float)r2c));
-            r2i = fmaf(r2i, fmaf(-(float)r2c, r2i, 1.0f), r2i);
+            float r2i, ri;
+            asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r2i) : "f"((float)e.r2));
+            asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(ri) : "f"((float)e.r2));
+            r2i = fmaf(r2i, fmaf(-(float)e.r2, r2i, 1.0f), r2i);
             const float p = r2i * r2i;
             const float pe = fmaf(r2i, r2i, -p);                  // exact error of the square
             r6inv = (Real)fmaf(p, r2i, pe * r2i);                // r2i^3 rounded once
             r2inv = (Real)r2i;
-            rinv = (Real)rsqrtf((float)r2c);
+            rinv = (Real)ri;
         } else {
-            rinv = (Real)(1.0 / sqrt((double)r2c));
+            rinv = (Real)(1.0 / sqrt((double)e.r2));
             r2inv = rinv * rinv;
             r6inv = r2inv * r2inv * r2inv;
         }
@@ -626,32 +711,60 @@ __device__ void nl_step_item(const SysDev &S, int k0, int par, int *viol, const 
             // Eq. 4 path for a pair with a changing bead: each end state's
             // Lennard-Jones at s = r^2 + delta (1 - its weight), force/r =
             // s^-4 (12 C12 s^-3 - 6 C6); the reaction field stays linear
-            const Real ia = (Real)1 / (r2c + dsc * lam), ib = (Real)1 / (r2c + dsc * ((Real)1 - lam));
+            const Real ia = (Real)1 / (e.r2 + dsc * lam), ib = (Real)1 / (e.r2 + dsc * ((Real)1 - lam));
             const Real ia3 = ia * ia * ia, ib3 = ib * ib * ib;
-            const Real lja = fmr(ca.x, ia3, -ca.y) * (ia3 * ia), ljb = fmr(cb.x, ib3, -cb.y) * (ib3 * ib);
+            const Real lja = fmr(ca.f12, ia3, -ca.f6) * (ia3 * ia), ljb = fmr(cb.f12, ib3, -cb.f6) * (ib3 * ib);
             fs = fmr((Real)1 - lam, lja, fmr(lam, ljb, qq * fmr(rinv, r2inv, -krf2)));
         }
-        fs = in ? fs : (Real)0;
-        ax = fmr(fs, dx, ax); ay = fmr(fs, dy, ay); az = fmr(fs, dz, az);
-        if (PC) { wx = fmr(fs * dx, dx, wx); wy = fmr(fs * dy, dy, wy); wz = fmr(fs * dz, dz, wz); }
+        fs = e.in ? fs : (Real)0;
+        ax = fmr(fs, e.x, ax); ay = fmr(fs, e.y, ay); az = fmr(fs, e.z, az);
+        if (PC) { wx = fmr(fs * e.x, e.x, wx); wy = fmr(fs * e.y, e.y, wy); wz = fmr(fs * e.z, e.z, wz); }
     };
 
-    // column gl of the bead's list, rows 0 .. cnt - 1, in groups of 4: as
-    // soon as a row is summed, its register takes the position of the row
-    // 4 further on and the index of the row 8 further on, so every load has
-    // a whole group of pairs to arrive (entries past the end read slot 0)
+    // Column gl of the bead's list, rows 0 .. cnt - 1 in groups of 4 (the
+    // build pads a column to whole groups with the bead itself).  Two rows at
+    // a time: their positions' registers take the rows 4 further on as soon as
+    // the separations are known, and the index registers the group after, so
+    // every load has most of a group to arrive.
+    //
+    // What bounds the loop: the wavefronts of its gathers and table reads (about
+    // 22 per warp and row before, 14 of them the gather) and, next, its
+    // instructions (72 per entry before).  With 8-byte table entries, four
+    // indices per load, no branch per pair and no bounds test per row a step of
+    // the 1152-lipid bilayer takes 14.8 us without a trial (17.5 before), of
+    // the 4608-lipid one 46.8 (54), of the 128-lipid one 8.6 (12.2).
     const int rows = cnt;
-    auto idx = [&](int r) { return r < rows ? MDAS_IDX(C, ld_list(lst + (size_t)r * rs), n) : 0; };
+    unsigned long long aw = 0;
     for (int pass = 0;; ++pass) {
-        j0 = idx(4); j1 = idx(5); j2 = idx(6); j3 = idx(7);
+        const int4 *nxt = lst + rs;
+        if (4 < rows) j = rows4(nxt);
         for (int m = 0; m < rows; m += 4) {
-            pair(q0, true);          q0 = cur[j0]; j0 = idx(m + 8);
-            pair(q1, m + 1 < rows);  q1 = cur[j1]; j1 = idx(m + 9);
-            pair(q2, m + 2 < rows);  q2 = cur[j2]; j2 = idx(m + 10);
-            pair(q3, m + 3 < rows);  q3 = cur[j3]; j3 = idx(m + 11);
+            {
+                Sep a = cull(q0), b = cull(q1);
+                if (a.edge | b.edge) {
+                    if (a.edge) a.in = in_exact(q0);
+                    if (b.edge) b.in = in_exact(q1);
+                }
+                q0 = cur[j.x]; q1 = cur[j.y];
+                add(a); add(b);
+            }
+            {
+                Sep a = cull(q2), b = cull(q3);
+                if (a.edge | b.edge) {
+                    if (a.edge) a.in = in_exact(q2);
+                    if (b.edge) b.in = in_exact(q3);
+                }
+                q2 = cur[j.z]; q3 = cur[j.w];
+                nxt += rs;
+                if (m + 8 < rows) j = rows4(nxt);
+                add(a); add(b);
+            }
         }
         // this lane's share of the bead's bonded terms (partners staged by all
-        // lanes of the bead: wait for the copies, then the warp barrier)
+        // lanes of the bead: wait for the copies, then the warp barrier); the
+        // thermostat factor published beside this step is loaded meanwhile
+        if (F32 && pw != nullptr && pw->has_close && gl == 0 && valid)
+            aw = ld_relaxed64(&C.alpha_pack[sm.sid[il] < P.n_lipid_beads ? 0 : 1]);
         cp_async_wait_all();
         __syncwarp();
         if (valid && meta_lip(pi.w) >= 0) {
@@ -681,7 +794,7 @@ __device__ void nl_step_item(const SysDev &S, int k0, int par, int *viol, const 
         // item sees (a changed bead or a changed partner), the same sums again
         // with the new bead types, read past the L1 cache
         if (pw == nullptr || pass > 0 || !pw->has_trial) break;
-        if (t == 0) sm.redo = pipe_wait(S, *pw, k0 / NL_BEADS);
+        if (t == 0) sm.redo = pipe_wait(S, P.mark_words, *pw, k0 / NL_BEADS);
         g.sync();
         if (!sm.redo) break;
         __threadfence();
@@ -689,17 +802,20 @@ __device__ void nl_step_item(const SysDev &S, int k0, int par, int *viol, const 
         if (valid) pi = __ldcg(cur + k);
         tai = meta_ta(pi.w) * 16;
         tbi = meta_tb(pi.w) * 16;
+        charged = ((qrow >> meta_ta(pi.w)) | (ALCH ? qrow >> meta_tb(pi.w) : 0u)) & 1u;
         ax = ay = az = (Real)0;
         wx = wy = wz = (Real)0;
-        j0 = idx(0); j1 = idx(1); j2 = idx(2); j3 = idx(3);
-        q0 = __ldcg(cur + j0); q1 = __ldcg(cur + j1); q2 = __ldcg(cur + j2); q3 = __ldcg(cur + j3);
+        if (0 < rows) j = rows4(lst);
+        q0 = __ldcg(cur + j.x); q1 = __ldcg(cur + j.y); q2 = __ldcg(cur + j.z); q3 = __ldcg(cur + j.w);
     }
     Real e0 = 0, e1 = 0;
     Real kx = 0, ky = 0, kz = 0;               // PC: the bead's kinetic energy per axis
     if (valid && gl == 0) {
+        uint4 np = pi;
+        const int id = sm.sid[il];
         const Real f0 = ax, f1 = ay, f2 = az;
         const int grp = id < P.n_lipid_beads ? 0 : 1;
-        const Real a = pw != nullptr && pw->has_close ? alpha_beside_close<Real>(C, grp, *pw)
+        const Real a = pw != nullptr && pw->has_close ? alpha_beside_close<Real>(C, grp, *pw, aw)
                        : (F32 ? (Real)C.alpha_f[grp] : (Real)C.alpha[grp]);
         const Real dtm = F32 ? (Real)P.dt_over_mf : (Real)P.dt_over_m;
         V4 v = sm.svel[il];
@@ -715,7 +831,7 @@ __device__ void nl_step_item(const SysDev &S, int k0, int par, int *viol, const 
         }
         reinterpret_cast<V4 *>(S.vel)[id] = v;
         if (!(isfinite(v.x) && isfinite(v.y) && isfinite(v.z))) atomicOr(&C.err, ERR_NONFINITE);
-        uint4 np = pi;
+        if (KEEP) sm.svel[il] = v;             // for the item's next step
         if (F32) {
             np.x += (uint32_t)__float2int_rn((float)v.x * P.qdtf[0]);
             np.y += (uint32_t)__float2int_rn((float)v.y * P.qdtf[1]);
@@ -726,7 +842,8 @@ __device__ void nl_step_item(const SysDev &S, int k0, int par, int *viol, const 
             np.z += (uint32_t)(long long)rint((double)v.z * P.qdt[2]);
         }
         S.pos[id] = np;
-        nxt[k] = np;
+        S.lpos[(size_t)(par ^ 1) * n + k] = np;
+        if constexpr (KEEP) sm.keep.spos[il] = np;
         // displacement since the list build
         const uint4 xr = sm.sxref[il];
         const float ux = (float)(int)(np.x - xr.x) * qs0;
@@ -870,14 +987,14 @@ static __global__ void __launch_bounds__(GRP) k_nl_place(const SysDev *__restric
     const int2 bm = bmap[blockIdx.x];
     const SysDev &S = sys[bm.x];
     if (!S.c->nl_stale) return;
-    nl_place_item(S, bm.y, S.c->nl_par, Grp{(int)threadIdx.x, 1}, sm);
+    nl_place_item(S, bm.y, S.c->nl_par, NLB_BEADS, Grp{(int)threadIdx.x, 1}, sm);
 }
 
 template <int G>
 __global__ void __launch_bounds__(GRP) k_nl_build(const SysDev *__restrict__ sys, int n_sys) {
     __shared__ BuildSmem sm;
     const int w = threadIdx.x >> 5;
-    nl_build_dealt<G>(sys, n_sys, w * gridDim.x + blockIdx.x, (GRP / 32) * gridDim.x, threadIdx.x & 31, sm.w[w],
+    nl_build_dealt<G, NLB_BEADS>(sys, n_sys, w * gridDim.x + blockIdx.x, (GRP / 32) * gridDim.x, threadIdx.x & 31, sm.w[w],
                       [](const SysDev &S) { return S.c->nl_stale != 0; },
                       [](const SysDev &S) { return S.c->nl_par; });
 }
@@ -905,13 +1022,16 @@ void launch_nl_build_t(const LaunchCtx &L) {
 // waiting) closes the step and flags the list stale after a violation.
 template <typename Real, int LAM, int G>
 __global__ void __launch_bounds__(GRP, 8) k_nl_step(const SysDev *__restrict__ sys, const int2 *__restrict__ bmap) {
-    __shared__ StepSmem<Real, G> sm;
+    __shared__ StepSmem<Real, G, false> sm;
     __shared__ int last;
     const int2 bm = bmap[blockIdx.x];
     const SysDev &S = sys[bm.x];
     Counters &C = *S.c;
     const int par = C.nl_par;
-    nl_step_item<Real, LAM, G>(S, bm.y, par, &C.nl_viol, Grp{(int)threadIdx.x, 1}, sm);
+    const Grp g{(int)threadIdx.x, 1};
+    load_system<Real, G, false>(S, g, sm);
+    g.sync();
+    nl_step_item<Real, LAM, G, false>(bm.y, par, &C.nl_viol, g, sm);
     if (threadIdx.x == 0) {
         __threadfence();
         const unsigned nblk = (unsigned)((S.p->n + NL_BLOCK / G - 1) / (NL_BLOCK / G));
@@ -1057,9 +1177,15 @@ static __device__ bool grid_barrier_flag(RunSync *rs, BarState &bs, const RunArg
 
 // List build of every system whose flag is set; buffer (nl_par + b) & 1 holds
 // the current positions.  Three barriers.
+//
+// Tasks of NLB_FEW beads while the beads still give every warp of the grid at
+// most one such task (shorter chains per warp: 25 against 33 us for the
+// 128-lipid bilayer's task phase), of NLB_BEADS beyond (fewer walks over the
+// candidates).
 template <int NG>
-__device__ bool run_build(const RunArgs &a, int which, int s, int b, const Grp &g, int gid, int G, BuildSmem &sm,
-                          BarState &bs) {
+__device__ __noinline__ bool run_build(const RunArgs &a, int which, int s, int b, const Grp &g, int gid, int G, BuildSmem &sm,
+                                       BarState &bs) {
+    const bool few = a.n_bead * (BEAD_BLOCK / NLB_FEW) <= (GRP / 32) * G;
     for (int it = gid; it < a.n_bead; it += G) {
         const int2 bm = a.beadmap[it];
         const SysDev &S = a.sys[bm.x];
@@ -1069,14 +1195,15 @@ __device__ bool run_build(const RunArgs &a, int which, int s, int b, const Grp &
     for (int it = gid; it < a.n_lsort; it += G) {
         const int2 bm = a.lsortmap[it];
         const SysDev &S = a.sys[bm.x];
-        if (build_flag(*S.c, which, s)) nl_place_item(S, bm.y, (S.c->nl_par + b) & 1, g, sm);
+        if (build_flag(*S.c, which, s)) nl_place_item(S, bm.y, (S.c->nl_par + b) & 1, few ? NLB_FEW : NLB_BEADS, g, sm);
     }
     if (!grid_barrier(a.rs, bs)) return false;
     // one warp per task, consecutive tasks on different SMs
     const int w = g.t >> 5;
-    nl_build_dealt<NG>(a.sys, a.n_sys, w * G + gid, (GRP / 32) * G, g.t & 31, sm.w[w],
-                       [&](const SysDev &S) { return build_flag(*S.c, which, s) != 0; },
-                       [&](const SysDev &S) { return (S.c->nl_par + b) & 1; });
+    auto flag = [&](const SysDev &S) { return build_flag(*S.c, which, s) != 0; };
+    auto par = [&](const SysDev &S) { return (S.c->nl_par + b) & 1; };
+    if (few) nl_build_dealt<NG, NLB_FEW>(a.sys, a.n_sys, w * G + gid, (GRP / 32) * G, g.t & 31, sm.w[w], flag, par);
+    else nl_build_dealt<NG, NLB_BEADS>(a.sys, a.n_sys, w * G + gid, (GRP / 32) * G, g.t & 31, sm.w[w], flag, par);
     return grid_barrier(a.rs, bs);
 }
 
@@ -1105,6 +1232,27 @@ static __device__ bool sys_barrier(SysBar *sb, unsigned base, unsigned &passes, 
     return *ok != 0;
 }
 
+// The list build of one system by its groups (partitioned mode; three
+// barriers); position buffer par.  Not inlined: a call per build costs
+// nothing, and the step's registers are not spilled around its code.
+template <int G>
+__device__ __noinline__ bool part_build(const RunArgs &a, const SysRange &R, const SysDev &S, int par, int lg, const Grp &g,
+                                        BuildSmem &bsm, SysBar *sb, unsigned base, unsigned &passes, int *ok) {
+    const int ng = R.ng;
+    auto bar = [&]() { return sys_barrier(sb, base, passes, ng, a.rs, g, ok); };
+    for (int it = lg; it < R.bdn; it += ng) nl_count_item(S, a.beadmap[R.bd0 + it].y, g);
+    if (!bar()) return false;
+    for (int it = lg; it < R.lsn; it += ng) nl_place_item(S, a.lsortmap[R.ls0 + it].y, par, NLB_BEADS, g, bsm);
+    if (!bar()) return false;
+    {
+        // the system's list-build tasks over its groups' warps in turn
+        const int T = __ldcg(&S.c->nbtask), w = g.t >> 5;
+        for (int t = w * ng + lg; t < T; t += (GRP / 32) * ng)
+            nl_build_task<G, NLB_BEADS>(S, t, par, g.t & 31, bsm.w[w]);
+    }
+    return bar();
+}
+
 // Partitioned mode (a batch of several systems whose step items do not all
 // fit the groups at once): every group belongs to one system and the
 // systems' groups advance independently, each system with barriers over its
@@ -1114,7 +1262,7 @@ static __device__ bool sys_barrier(SysBar *sb, unsigned base, unsigned &passes, 
 // alone; while one system's groups wait at a barrier, other systems' groups
 // on the same SM keep working.
 template <typename Real, int LAM, int G>
-__device__ void run_partitioned(const RunArgs &a, int gid, const Grp &g, StepSmem<Real, G> &ssm, BuildSmem &bsm,
+__device__ void run_partitioned(const RunArgs &a, int gid, const Grp &g, StepSmem<Real, G, false> &ssm, BuildSmem &bsm,
                                 TrialSmem &tsm, int *ok) {
     const int q = a.gsys[gid];
     if (q < 0) return;
@@ -1126,20 +1274,7 @@ __device__ void run_partitioned(const RunArgs &a, int gid, const Grp &g, StepSme
     unsigned base = 0, passes = 0;
     if (g.t == 0) base = *(volatile const unsigned *)&sb->base;
     auto bar = [&]() { return sys_barrier(sb, base, passes, ng, a.rs, g, ok); };
-    // the list build of this system (three barriers); position buffer par
-    auto build = [&](int par) {
-        for (int it = lg; it < R.bdn; it += ng) nl_count_item(S, a.beadmap[R.bd0 + it].y, g);
-        if (!bar()) return false;
-        for (int it = lg; it < R.lsn; it += ng) nl_place_item(S, a.lsortmap[R.ls0 + it].y, par, g, bsm);
-        if (!bar()) return false;
-        {
-            // the system's list-build tasks over its groups' warps in turn
-            const int T = __ldcg(&C.nbtask), w = g.t >> 5;
-            for (int t = w * ng + lg; t < T; t += (GRP / 32) * ng)
-                nl_build_task<G, false>(S, t, par, g.t & 31, bsm.w[w]);
-        }
-        return bar();
-    };
+    auto build = [&](int par) { return part_build<G>(a, R, S, par, lg, g, bsm, sb, base, passes, ok); };
     bool tab = true;                           // the pair tables must be (re)loaded into shared memory
     if (*(volatile const int *)&C.nl_stale) {  // lists made stale outside the kernel
         if (!build(C.nl_par & 1)) return;
@@ -1149,8 +1284,12 @@ __device__ void run_partitioned(const RunArgs &a, int gid, const Grp &g, StepSme
     constexpr bool PC = LAM == 3;
     for (int s = 0; s < a.n_steps; ++s) {
         for (int it = lg; it < R.nln; it += ng) {
-            nl_step_item<Real, LAM, G>(S, a.nlmap[R.nl0 + it].y, (C.nl_par + s) & 1, &C.nl_violp[s % 3], g, ssm, tab);
-            tab = false;
+            if (tab) {
+                load_system<Real, G, false>(S, g, ssm);
+                g.sync();
+                tab = false;
+            }
+            nl_step_item<Real, LAM, G, false>(a.nlmap[R.nl0 + it].y, (C.nl_par + s) & 1, &C.nl_violp[s % 3], g, ssm);
         }
         // the flag of step s + 1 (last read at step s - 2, before the previous barrier)
         if (lg == 0 && g.t == 0) {
@@ -1204,14 +1343,14 @@ __device__ void run_partitioned(const RunArgs &a, int gid, const Grp &g, StepSme
 // The partitioned mode as a kernel of its own (same launch shape as
 // k_md_run, so either runs resident on the same device).
 template <typename Real, int LAM, int G>
-__global__ void __launch_bounds__(RUN_THREADS, 1) k_md_part(RunArgs a) {
+__global__ void __launch_bounds__(RUN_THREADS, 1) k_md_part(const __grid_constant__ RunArgs a) {
     extern __shared__ __align__(16) unsigned char dsm[];
     __shared__ int gok[RUN_GROUPS];
     const int group = threadIdx.x / GRP;
     const Grp g{(int)threadIdx.x % GRP, 1 + group};
     const int gid = group * gridDim.x + blockIdx.x;
-    unsigned char *gsm = dsm + group * group_smem<Real, G>();
-    run_partitioned<Real, LAM, G>(a, gid, g, *reinterpret_cast<StepSmem<Real, G> *>(gsm), *reinterpret_cast<BuildSmem *>(gsm),
+    unsigned char *gsm = dsm + group * group_smem<Real, G, false>();
+    run_partitioned<Real, LAM, G>(a, gid, g, *reinterpret_cast<StepSmem<Real, G, false> *>(gsm), *reinterpret_cast<BuildSmem *>(gsm),
                                *reinterpret_cast<TrialSmem *>(gsm), &gok[group]);
 }
 
@@ -1230,20 +1369,22 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_md_part(RunArgs a) {
 // again with the new types.  The arithmetic is that of the sequential order
 // (close and trial after the step's barrier, then a second barrier), which
 // runs otherwise.  Per step: items, barrier, list builds called for by the
-// step's displacements.
-template <typename Real, int LAM, int G>
-__global__ void __launch_bounds__(RUN_THREADS, 1) k_md_run(RunArgs a) {
+// step's displacements.  The mode is a template parameter (PIPE; the host
+// decides it by md_run_pipe): each kernel asks for its own shared memory, and
+// the other mode's code takes no registers.
+template <typename Real, int LAM, int G, bool PIPE>
+__global__ void __launch_bounds__(RUN_THREADS, 1) k_md_run(const __grid_constant__ RunArgs a) {
     extern __shared__ __align__(16) unsigned char dsm[];
     const int group = threadIdx.x / GRP;
     const Grp g{(int)threadIdx.x % GRP, 1 + group};
     // consecutive items go to different SMs
     const int ngr = gridDim.x * RUN_GROUPS, gid = group * gridDim.x + blockIdx.x;
-    unsigned char *gsm = dsm + group * group_smem<Real, G>();
-    StepSmem<Real, G> &ssm = *reinterpret_cast<StepSmem<Real, G> *>(gsm);
+    unsigned char *gsm = dsm + group * group_smem<Real, G, PIPE>();
+    StepSmem<Real, G, PIPE> &ssm = *reinterpret_cast<StepSmem<Real, G, PIPE> *>(gsm);
     BuildSmem &bsm = *reinterpret_cast<BuildSmem *>(gsm);
     TrialSmem &tsm = *reinterpret_cast<TrialSmem *>(gsm);
 
-    const bool pipe = a.n_nl + (TRIAL_PARTS + 1) * a.n_sys <= ngr;
+    constexpr bool pipe = PIPE;
     const int dg = ngr - 1 - gid;                // the last gids: trial parts, then closes
     const int ptrial = pipe && dg < TRIAL_PARTS * a.n_sys ? dg : -1;
     const int pclose = pipe && ptrial < 0 && dg < (TRIAL_PARTS + 1) * a.n_sys ? dg - TRIAL_PARTS * a.n_sys : -1;
@@ -1268,7 +1409,8 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_md_run(RunArgs a) {
             for (int q = blockIdx.x; q < a.n_sys; q += gridDim.x)
                 if (a.sys[q].c->nl_stale) a.sys[q].c->nl_builds++;
     }
-    int tab_sys = -1;                          // system whose tables the group holds
+    int tab_sys = -1;                          // system whose data the group's scratch holds
+    bool kept = false;                         // (overlapped mode) and the item's beads
     for (int s = 0; s < a.n_steps; ++s) {
         // a trial after step s - 1: the ordinal o of that trial in this launch
         const bool tprev = s > 0 && a.swap_every > 0 && (s + a.trial_off) % a.swap_every == 0;
@@ -1283,9 +1425,14 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_md_run(RunArgs a) {
                 pw.has_trial = tprev;
                 pw.T = trial0 + (unsigned long long)o;
                 pw.mark_target = mark0 + (unsigned)(TRIAL_PARTS * (o + 1));
-                nl_step_item<Real, LAM, G>(S, bm.y, (S.c->nl_par + s) & 1, &S.c->nl_violp[s % 3], g, ssm,
-                                        bm.x != tab_sys, &pw);
-                tab_sys = bm.x;
+                if (tab_sys < 0) {
+                    load_system<Real, G, PIPE>(S, g, ssm);
+                    g.sync();
+                    tab_sys = bm.x;
+                    kept = false;
+                }
+                nl_step_item<Real, LAM, G, PIPE>(bm.y, (S.c->nl_par + s) & 1, &S.c->nl_violp[s % 3], g, ssm, &pw, kept);
+                kept = true;
             } else if (ptrial >= 0 && tprev) {
                 const SysDev &S = a.sys[ptrial / TRIAL_PARTS];
                 trial_nl_part<G>(S, ptrial % TRIAL_PARTS, (S.c->nl_par + s) & 1, g, tsm, true);
@@ -1297,9 +1444,12 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_md_run(RunArgs a) {
             for (int it = gid; it < a.n_nl; it += ngr) {
                 const int2 bm = a.nlmap[it];
                 const SysDev &S = a.sys[bm.x];
-                nl_step_item<Real, LAM, G>(S, bm.y, (S.c->nl_par + s) & 1, &S.c->nl_violp[s % 3], g, ssm,
-                                        bm.x != tab_sys);
-                tab_sys = bm.x;
+                if (bm.x != tab_sys) {
+                    load_system<Real, G, PIPE>(S, g, ssm);
+                    g.sync();
+                    tab_sys = bm.x;
+                }
+                nl_step_item<Real, LAM, G, PIPE>(bm.y, (S.c->nl_par + s) & 1, &S.c->nl_violp[s % 3], g, ssm);
             }
         }
         // the flag of step s + 1 (last read at step s - 2, before the previous barrier)
@@ -1386,6 +1536,12 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_md_run(RunArgs a) {
         }
 }
 
+// Whether a launch of n_blocks persistent blocks over n_items step items of
+// n_sys systems runs in overlapped mode (see k_md_run).
+inline bool md_run_pipe(int n_items, int n_sys, int n_blocks) {
+    return n_items + (TRIAL_PARTS + 1) * n_sys <= n_blocks * RUN_GROUPS;
+}
+
 template <typename Real, int LAM, int G>
 static cudaError_t run_launch(const LaunchCtx &L, int n_steps, int swap_every, int trial_off, int lam_M,
                               int lam_off, double dlam, RunSync *rs, int n_blocks) {
@@ -1405,35 +1561,37 @@ static cudaError_t run_launch(const LaunchCtx &L, int n_steps, int swap_every, i
     a.n_steps = n_steps; a.swap_every = swap_every; a.trial_off = trial_off; a.rs = rs;
     a.lam_M = lam_M; a.lam_off = lam_off; a.dlam = dlam;
     void *args[] = {&a};
-    const void *fn = a.gsys ? (const void *)k_md_part<Real, LAM, G> : (const void *)k_md_run<Real, LAM, G>;
-    return cudaLaunchCooperativeKernel(fn, dim3(n_blocks), dim3(RUN_THREADS), args, RUN_GROUPS * group_smem<Real, G>(),
+    const bool pipe = !a.gsys && md_run_pipe(a.n_nl, a.n_sys, n_blocks);
+    const void *fn = a.gsys ? (const void *)k_md_part<Real, LAM, G>
+                     : pipe ? (const void *)k_md_run<Real, LAM, G, true> : (const void *)k_md_run<Real, LAM, G, false>;
+    return cudaLaunchCooperativeKernel(fn, dim3(n_blocks), dim3(RUN_THREADS), args,
+                                       RUN_GROUPS * (pipe ? group_smem<Real, G, true>() : group_smem<Real, G, false>()),
                                        L.stream);
 }
 
+// Shared-memory limits of the three kernels, and whether a block of each fits
+// on an SM.  No more shared memory than a block needs: the rest of the SM's
+// 256 KB stays L1 cache for the step's position gathers.
 template <typename Real, int LAM, int G>
 static cudaError_t run_setup(int *blocks_per_sm) {
-    const size_t smem = RUN_GROUPS * group_smem<Real, G>();
-    cudaError_t e = cudaFuncSetAttribute(k_md_run<Real, LAM, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_md_part<Real, LAM, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    {
-        // no more shared memory than the block needs: the rest of the SM's
-        // 256 KB stays L1 cache for the step's position gathers
-        int dev = 0, maxsm = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-        const int carve = maxsm > 0 ? std::min(100, (int)(100.0 * (double)(smem + 4096) / maxsm) + 1) : 100;
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_md_run<Real, LAM, G>, cudaFuncAttributePreferredSharedMemoryCarveout, carve);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_md_part<Real, LAM, G>, cudaFuncAttributePreferredSharedMemoryCarveout, carve);
+    const struct { const void *fn; size_t smem; } kernels[] = {
+        {(const void *)k_md_run<Real, LAM, G, true>, RUN_GROUPS * group_smem<Real, G, true>()},
+        {(const void *)k_md_run<Real, LAM, G, false>, RUN_GROUPS * group_smem<Real, G, false>()},
+        {(const void *)k_md_part<Real, LAM, G>, RUN_GROUPS * group_smem<Real, G, false>()}};
+    int dev = 0, maxsm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    *blocks_per_sm = 1 << 20;
+    for (const auto &k : kernels) {
+        cudaError_t e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);
+        const int carve = maxsm > 0 ? std::min(100, (int)(100.0 * (double)(k.smem + 4096) / maxsm) + 1) : 100;
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k.fn, cudaFuncAttributePreferredSharedMemoryCarveout, carve);
+        int per = 0;
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k.fn, RUN_THREADS, k.smem);
+        if (e != cudaSuccess) return e;
+        *blocks_per_sm = std::min(*blocks_per_sm, per);
     }
-    if (e != cudaSuccess) return e;
-    int per_part = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_md_run<Real, LAM, G>, RUN_THREADS, smem);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_part, k_md_part<Real, LAM, G>, RUN_THREADS, smem);
-    if (e == cudaSuccess) *blocks_per_sm = std::min(*blocks_per_sm, per_part);
-    return e;
+    return cudaSuccess;
 }
 
 // Blocks of the persistent kernel on this device: one per SM when a block
