@@ -617,16 +617,22 @@ int trial_path_of(const Batch &b, int) {
     return MDAS_TRIALS_SEQUENTIAL;
 }
 
-// n exchange trials of every system of a batch, one after another from the
-// pair lists (the trial the persistent kernel runs after an MD step): one
-// launch per trial with every system's 16 parts, no speculation and no
-// host round trip; the lists are built first where stale.
+// The lipids of a batch's largest system.
+int max_lipids(const Batch &b) {
+    int n = 0;
+    for (const mdas_system *x : b.sys) n = std::max(n, x->n_lip);
+    return n;
+}
+
+// n exchange trials of every system of a batch, with the result of one after
+// another, from the pair lists, in a few launches per chunk of trials and with
+// no host round trip; the lists are built first where stale.
 mdas_status run_trials_nl(mdas_system *s, Batch &b, int n) {
     mdas_status st = lists_for_shape(s, b);
     if (st != MDAS_OK) return st;
     LaunchCtx L = b.ctx();
     launch_nl_build(L);
-    for (int t = 0; t < n; ++t) launch_trial_nl(L);
+    launch_swap_trials(L, n, max_lipids(b));
     for (auto *x : b.sys) x->cells_valid = false;   // the cell-ordered copy keeps the old types
     CK(cudaGetLastError());
     return check_err(s, b);
@@ -885,7 +891,7 @@ mdas_status mdas_create_system(const mdas_system_desc *d, mdas_system **out) {
         {(void **)&H.spos, 16ull * nslot}, {(void **)&H.bforce, vsz * nslot},
         {(void **)&H.ke_part, 16ull * P.n_cells}, {(void **)&H.bpart, 24ull * nbb}, {(void **)&H.epart, 32ull * P.n_cells},
         {(void **)&H.pos_snap, 16ull * n}, {(void **)&H.vel_snap, vsz * n},
-        {(void **)&H.ltype_snap, 4ull * std::max(nl, 1)},
+        {(void **)&H.thead, 4ull * std::max(nl, 1)}, {(void **)&H.tnext, 8ull * CHAIN_MAX},
         {(void **)&H.tprop, 16ull * MAX_ROUND_TRIALS}, {(void **)&H.tu, 8ull * MAX_ROUND_TRIALS},
         {(void **)&H.tdE, 8ull * 9 * MAX_ROUND_TRIALS}, {(void **)&H.tstate, 4ull * MAX_ROUND_TRIALS},
         {(void **)&H.conflict, 4ull * MAX_ROUND_TRIALS * (MAX_ROUND_TRIALS / 32)},
@@ -1072,7 +1078,7 @@ mdas_status mdas_mutation_trials(mdas_system *s, int32_t n_trials, const double 
     mdas_status st = build_cells(s, b);
     if (st != MDAS_OK) return st;
     LaunchCtx L = b.ctx();
-    launch_mutation_trials(L, n_trials);
+    launch_mutation_trials(L, n_trials, s->n_lip);
     s->kernel_launches += 1;
     Counters c1;
     CK(cudaMemcpyAsync(&c1, s->hs.c, sizeof(Counters), cudaMemcpyDeviceToHost, s->stream));
@@ -1952,12 +1958,12 @@ size_t arena_estimate(const mdas_system_desc *d) {
     size_t t = sizeof(Params) + sizeof(Counters) + 16 * n + vsz * n + 24 * n + 8 * std::max(d->n_lipids, 1) +
                8 * nc + 24 * nc * capc + vsz * nc * capc + 4 * n + 16 * nc + 24 * nbb + 32 * nc + 16 * n + vsz * n +
                (16 + 8 + 72 + 4 + 128 + 64) * (size_t)MAX_ROUND_TRIALS + sizeof(TrialRec) * (size_t)LOG_CAP + 512 +
-               32 * MAX_DRAW_STEPS + 24 * n + 16 * std::max(d->n_lipids, 1) + 16 * RDF_MAX_BINS + 8;
+               32 * MAX_DRAW_STEPS + 8 * CHAIN_MAX + 24 * n + 16 * std::max(d->n_lipids, 1) + 16 * RDF_MAX_BINS + 8;
     const ListDims ld = list_dims(d, shrink);
     t += 12ull * ld.n_lcells + 4ull * ld.n_lcells * ld.lcapc + 4 * n + 4 * n + 32 * n + 16 * n + 4ull * NL_LANES_MAX * n +
          4ull * ld.lcap * ld.npad + 4ull * NL_PART * n + 8ull * ((n + NL_BEADS_MIN - 1) / NL_BEADS_MIN / 32 + 1) +
          8ull * (n / NLB_FEW + ld.n_lcells + 1);
-    return t + 52 * 256;
+    return t + 53 * 256;
 }
 
 }  // namespace

@@ -34,6 +34,8 @@ __host__ __device__ constexpr int nl_build_tasks(int beads, int run) { return (b
 constexpr int CELLS_PER_SORT_BLOCK = 4;
 constexpr int LOG_CAP = 65536;         // trial records kept per system
 constexpr int MAX_ROUND_TRIALS = 1024; // trials per batched swap evaluation
+constexpr int CHAIN_MAX = 256;         // trials of a chunk that runs in order, many per launch,
+constexpr int CHAIN_MIN = 16;          // and the fewest that are evaluated ahead
 constexpr int MAX_PAIRS = 64;
 constexpr int DE_GROUPS = 9;           // blocks that share the energy change of one batched trial
 constexpr int TRIAL_PARTS = 16;        // 128-thread parts of one trial over the pair list
@@ -235,12 +237,12 @@ struct SysDev {
     double *bpart;                     // [n_bead_blocks * 3] bond, angle, kinetic energies (FP64)
     uint4 *pos_snap;
     void *vel_snap;
-    int *ltype_snap;
     // batched exchange trials
     int4 *tprop;                       // a, b, type a, type b
     double *tu, *tdE;
     int *tstate;                       // 0 pending, 1 resolved
     uint32_t *conflict;                // [MAX_ROUND_TRIALS * MAX_ROUND_TRIALS / 32]
+    int *thead, *tnext;                // trials of a chunk by lipid: [n_lip] first node, [2 CHAIN_MAX] next node
     int4 *lbox;                        // per-lipid box: centre (x,y,z), unused
     int4 *lhalf;                       // per-lipid half widths
     TrialRec *log;                     // [LOG_CAP]
@@ -405,7 +407,9 @@ void launch_mdas_accept(const LaunchCtx &L);
 void launch_mdas_restore(const LaunchCtx &L);
 void launch_snapshot(const LaunchCtx &L);
 void launch_delta_energy(const LaunchCtx &L, int n_changed_lipids);
-void launch_mutation_trials(const LaunchCtx &L, int n);
+// n trials of every system in order, many per launch; max_lip: lipids of the largest system
+void launch_swap_trials(const LaunchCtx &L, int n, int max_lip);       // over the pair lists (valid lists)
+void launch_mutation_trials(const LaunchCtx &L, int n, int max_lip);   // over the cells (a current cell list)
 // the work term of the lambda step l0 -> l1 from the pair list (valid lists)
 void launch_mdas_dE_nl(const LaunchCtx &L, double l0, double l1, double dlambda);
 void launch_head_rdf(const SysDev *dsys, int n_lip, int lt_sel, int head_k, double r_max, int n_bins, uint4 *info,

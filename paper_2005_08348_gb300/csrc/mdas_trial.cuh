@@ -63,6 +63,98 @@ __device__ inline double group_sum(double v, const Grp &g, double *sh) {
     return s;
 }
 
+// The beads that an exchange of the types (ta, tb) of lipids a and b changes,
+// and where their list entries begin in the trial's sequence of entries (beads
+// in order, columns in order within a bead), into sm; by one warp.  It loads,
+// for the beads of both lipids at once, their list slots, then their positions
+// and row counts, and scans the row counts itself.  mark(slot): called for
+// every changed bead.
+template <int G, class Mark>
+__device__ __forceinline__ void trial_beads(const SysDev &S, int a, int b, int ta, int tb, const uint4 *cur, int lane,
+                                            TrialSmem &sm, Mark mark) {
+    const Params &P = *S.p;
+    // lane (side, k): local index k of lipid a (side 0) or b (side 1)
+    const int bpl = P.bpl;
+    const int side = lane >= bpl, k = side ? lane - bpl : lane;
+    const bool valid = lane < 2 * bpl;
+    const int id = (side ? b : a) * bpl + k;
+    const int kk = valid ? MDAS_IDX(*S.c, S.lk[id], P.n) : 0;
+    const uint4 pk = cur[kk];
+    int cn[G];
+#pragma unroll
+    for (int c = 0; c < G; ++c) cn[c] = S.nl_n[(size_t)kk * G + c];
+    const bool null_trial = (a == b) || (ta == tb);
+    const int bo = P.lbt[(side ? tb : ta) * 16 + k], bn = P.lbt[(side ? ta : tb) * 16 + k];
+    const bool ch = valid && !null_trial && bo != bn;
+    const unsigned bal = __ballot_sync(0xffffffffu, ch);
+    int tot = 0;
+#pragma unroll
+    for (int c = 0; c < G; ++c) tot += cn[c];
+    if (!ch) tot = 0;
+    int inc = tot;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, inc, d);
+        if (lane >= d) inc += x;
+    }
+    if (ch) {
+        mark(kk);
+        const int o = __popc(bal & ((1u << lane) - 1u));
+        sm.chg_id[o] = id;
+        sm.chg_k[o] = kk;
+        sm.chg_pos[o] = pk;
+        sm.chg_old[o] = bo;
+        sm.chg_new[o] = bn;
+        int run = inc - tot;
+#pragma unroll
+        for (int c = 0; c < G; ++c) {
+            sm.it_beg[G * o + c] = run;
+            run += cn[c];
+        }
+    }
+    if (lane == 31) {
+        const int nc = __popc(bal);
+        sm.nchg = nc;
+        sm.it_beg[G * nc] = inc;
+        sm.m = (int)(bal & ((1u << bpl) - 1u));   // local indices whose bead type changes
+        sm.ta = ta;
+        sm.tb = tb;
+    }
+}
+
+// Energy change of entry f of the trial in sm (0 outside the cutoff; a pair of
+// two changed beads counts once, by the lower id).  seen(slot): called with the
+// partner's list slot before its position is loaded; near(lipid): with the
+// lipid of a partner inside the cutoff (-1: water).
+template <int G, class Seen, class Near>
+__device__ __forceinline__ double trial_entry(const SysDev &S, int a, int b, const uint4 *cur, const TrialSmem &sm, int f,
+                                              Seen seen, Near near) {
+    const Params &P = *S.p;
+    int lo = 0, hi = sm.nchg * G - 1;         // the (bead, column) holding entry f
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (sm.it_beg[mid] <= f) lo = mid; else hi = mid - 1;
+    }
+    const int ci = lo / G, q = lo % G, row = f - sm.it_beg[lo];
+    const int kj = MDAS_IDX(*S.c, S.nl[nl_at<G>(P.npad, sm.chg_k[ci], row, q)], P.n);
+    seen(kj);
+    const uint4 pi = sm.chg_pos[ci], pj = __ldcg(cur + kj);
+    const int ix = (int)(pi.x - pj.x), iy = (int)(pi.y - pj.y), iz = (int)(pi.z - pj.z);
+    const float fx = (float)ix * P.qsf[0], fy = (float)iy * P.qsf[1], fz = (float)iz * P.qsf[2];
+    const float r2f = fx * fx + fy * fy + fz * fz;
+    if (!(r2f < P.rc2f) || r2f == 0.0f) return 0.0;
+    const int lj = meta_lip(pj.w), kjl = meta_k(pj.w);
+    near(lj);
+    const bool chj = (lj == a || lj == b) && ((sm.m >> kjl) & 1);
+    if (chj && lj * P.bpl + kjl < sm.chg_id[ci]) return 0.0;   // a changed pair once, by the lower id
+    const double ex = (double)ix * P.qs[0], ey = (double)iy * P.qs[1], ez = (double)iz * P.qs[2];
+    const double r2 = ex * ex + ey * ey + ez * ez;
+    if (r2 >= P.rc2) return 0.0;
+    const int old_j = meta_ta(pj.w);
+    const int new_j = chj ? (int)P.lbt[(lj == a ? sm.tb : sm.ta) * 16 + kjl] : old_j;
+    return pair_du(P, sm.chg_old[ci], old_j, sm.chg_new[ci], new_j, r2);
+}
+
 // Part p (of TRIAL_PARTS) of one exchange trial from the pair list (valid
 // whenever an MD step has just run), by one 128-thread group.  The trial's
 // items are (changed bead, list column, row); part p takes every
@@ -70,11 +162,6 @@ __device__ inline double group_sum(double v, const Grp &g, double *sh) {
 // Every list holds all partners closer than rc, so the dE is the same sum as
 // over the 27 cells.  The last part to finish (a ticket) adds the part sums
 // in order, takes the Metropolis decision and applies it.
-//
-// Latency: one warp loads, for the beads of both lipids at once, their list
-// slots with the two lipid types, then their positions and list row counts;
-// it scans the row counts itself, so the entries start after one group
-// barrier.
 //
 // With mark set (the trial runs beside the next MD step), the parts set, in
 // bitmap T & 1, the bit of every step item (NL_BEADS list slots) that holds a
@@ -84,7 +171,7 @@ __device__ inline double group_sum(double v, const Grp &g, double *sh) {
 // (its last readers finished before this trial started).
 template <int G>
 __device__ inline void trial_nl_part(const SysDev &S, int p, int par, const Grp &g, TrialSmem &sm, bool mark) {
-    constexpr int NL_G = G, NL_BEADS = NL_BLOCK / G;
+    constexpr int NL_BEADS = NL_BLOCK / G;
     const Params &P = *S.p;
     Counters &C = *S.c;
     const int t = g.t, lane = t & 31;
@@ -94,87 +181,15 @@ __device__ inline void trial_nl_part(const SysDev &S, int p, int par, const Grp 
     const uint4 *cur = S.lpos + (size_t)par * P.n;
     const int words = P.mark_words;
     unsigned *const mk = S.tmark + (size_t)(T & 1) * words;
+    auto mark_item = [&](int k) { atomicOr(&mk[k / NL_BEADS / 32], 1u << (k / NL_BEADS % 32)); };
     for (int x = p * GRP + t; x < words; x += TRIAL_PARTS * GRP) S.tmark[(size_t)((T + 1) & 1) * words + x] = 0;
-    if (t < 32) {
-        // lane (side, k): local index k of lipid a (side 0) or b (side 1)
-        const int bpl = P.bpl;
-        const int side = lane >= bpl, k = side ? lane - bpl : lane;
-        const bool valid = lane < 2 * bpl;
-        const int id = (side ? b : a) * bpl + k;
-        const int kk = valid ? MDAS_IDX(*S.c, S.lk[id], P.n) : 0;
-        const int ta = S.ltype[a], tb = S.ltype[b];
-        const uint4 pk = cur[kk];
-        int cn[NL_G];
-#pragma unroll
-        for (int c = 0; c < NL_G; ++c) cn[c] = S.nl_n[(size_t)kk * NL_G + c];
-        const bool null_trial = (a == b) || (ta == tb);
-        const int bo = P.lbt[(side ? tb : ta) * 16 + k], bn = P.lbt[(side ? ta : tb) * 16 + k];
-        const bool ch = valid && !null_trial && bo != bn;
-        const unsigned bal = __ballot_sync(0xffffffffu, ch);
-        // entries of the changed beads in lane order, columns in order within
-        // a bead: exclusive offsets by one warp scan
-        int tot = 0;
-#pragma unroll
-        for (int c = 0; c < NL_G; ++c) tot += cn[c];
-        if (!ch) tot = 0;
-        int inc = tot;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const int x = __shfl_up_sync(0xffffffffu, inc, d);
-            if (lane >= d) inc += x;
-        }
-        if (ch) {
-            if (mark && p == 0) atomicOr(&mk[kk / NL_BEADS / 32], 1u << (kk / NL_BEADS % 32));
-            const int o = __popc(bal & ((1u << lane) - 1u));
-            sm.chg_id[o] = id;
-            sm.chg_k[o] = kk;
-            sm.chg_pos[o] = pk;
-            sm.chg_old[o] = bo;
-            sm.chg_new[o] = bn;
-            int run = inc - tot;
-#pragma unroll
-            for (int c = 0; c < NL_G; ++c) {
-                sm.it_beg[NL_G * o + c] = run;
-                run += cn[c];
-            }
-        }
-        if (lane == 31) {
-            const int nc = __popc(bal);
-            sm.nchg = nc;
-            sm.it_beg[NL_G * nc] = inc;
-            sm.m = (int)(bal & ((1u << bpl) - 1u));   // local indices whose bead type changes
-            sm.ta = ta;
-            sm.tb = tb;
-        }
-    }
+    if (t < 32) trial_beads<G>(S, a, b, S.ltype[a], S.ltype[b], cur, lane, sm, [&](int k) { if (mark && p == 0) mark_item(k); });
     g.sync();
-    const int nc = sm.nchg, nit = nc * NL_G, m = sm.m, ta = sm.ta, tb = sm.tb;
-    const int total = sm.it_beg[nit];
+    const int nc = sm.nchg, ta = sm.ta, tb = sm.tb;
+    const int total = sm.it_beg[nc * G];
     double acc = 0.0;
-    for (int f = p + TRIAL_PARTS * t; f < total; f += TRIAL_PARTS * GRP) {
-        int lo = 0, hi = nit - 1;                 // the item holding entry f
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (sm.it_beg[mid] <= f) lo = mid; else hi = mid - 1;
-        }
-        const int ci = lo / NL_G, q = lo % NL_G, row = f - sm.it_beg[lo];
-        const int kj = MDAS_IDX(*S.c, S.nl[nl_at<NL_G>(P.npad, sm.chg_k[ci], row, q)], P.n);
-        if (mark) atomicOr(&mk[kj / NL_BEADS / 32], 1u << (kj / NL_BEADS % 32));
-        const uint4 pi = sm.chg_pos[ci], pj = cur[kj];
-        const int ix = (int)(pi.x - pj.x), iy = (int)(pi.y - pj.y), iz = (int)(pi.z - pj.z);
-        const float fx = (float)ix * P.qsf[0], fy = (float)iy * P.qsf[1], fz = (float)iz * P.qsf[2];
-        const float r2f = fx * fx + fy * fy + fz * fz;
-        if (!(r2f < P.rc2f) || r2f == 0.0f) continue;
-        const int lj = meta_lip(pj.w), kjl = meta_k(pj.w);
-        const bool chj = (lj == a || lj == b) && ((m >> kjl) & 1);
-        if (chj && lj * P.bpl + kjl < sm.chg_id[ci]) continue;     // a changed pair once, by the lower id
-        const double ex = (double)ix * P.qs[0], ey = (double)iy * P.qs[1], ez = (double)iz * P.qs[2];
-        const double r2 = ex * ex + ey * ey + ez * ez;
-        if (r2 >= P.rc2) continue;
-        const int old_j = meta_ta(pj.w);
-        const int new_j = chj ? (int)P.lbt[(lj == a ? tb : ta) * 16 + kjl] : old_j;
-        acc += pair_du(P, sm.chg_old[ci], old_j, sm.chg_new[ci], new_j, r2);
-    }
+    for (int f = p + TRIAL_PARTS * t; f < total; f += TRIAL_PARTS * GRP)
+        acc += trial_entry<G>(S, a, b, cur, sm, f, [&](int k) { if (mark) mark_item(k); }, [](int) {});
     const double part = group_sum(acc, g, sm.sh);   // (its barriers order the group's marks)
     if (t == 0 && mark) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" :: "l"(&C.mark_seq) : "memory");
     if (t == 0) {

@@ -22,10 +22,14 @@ namespace mdas {
 // by the lower id only.  Candidates are culled in FP32 from exact integer
 // separations (those within float rounding of rc are decided in FP64); the
 // energies are FP64.  Types come from a functor of (meta, id) and a predicate
-// telling whether a neighbour is changed.
-template <class NewT, class Changed>
+// telling whether a neighbour is changed.  Of the cell's beads, those at first,
+// first + stride, ...; near(lipid) is called for every one inside the cutoff.
+struct NearNone {
+    __device__ void operator()(int) const {}
+};
+template <class NewT, class Changed, class Near = NearNone>
 __device__ double bead_delta(const SysDev &S, const Params &P, int i, uint4 pi, int old_i, int new_i, int slot,
-                             NewT newt, Changed changed) {
+                             NewT newt, Changed changed, int first = 0, int stride = 1, Near near = Near()) {
     const int nx = P.nc[0], ny = P.nc[1], nz = P.nc[2];
     const int cx = (int)(((unsigned long long)pi.x * (unsigned)nx) >> 32);
     const int cy = (int)(((unsigned long long)pi.y * (unsigned)ny) >> 32);
@@ -37,14 +41,15 @@ __device__ double bead_delta(const SysDev &S, const Params &P, int i, uint4 pi, 
     const uint32_t em = P.excl[ki];
     double acc = 0.0;
     const int e = cj * P.capc + S.cell_n[cj];
-    for (int p = cj * P.capc; p < e; ++p) {
-        const uint4 pj = S.spos[p];
+    for (int p = cj * P.capc + first; p < e; p += stride) {
+        const uint4 pj = __ldcg(&S.spos[p]);
         const int ix = (int)(pi.x - pj.x), iy = (int)(pi.y - pj.y), iz = (int)(pi.z - pj.z);
         const float fx = (float)ix * P.qsf[0], fy = (float)iy * P.qsf[1], fz = (float)iz * P.qsf[2];
         const float r2f = fx * fx + fy * fy + fz * fz;
         if (!(r2f < P.rc2f) || r2f == 0.0f) continue;
         const int j = S.sorted_id[p];
         if (j == i) continue;
+        near(meta_lip(pj.w));
         const bool chj = changed(pj.w, j);
         if (chj && j < i) continue;
         if (li >= 0 && meta_lip(pj.w) == li && ((em >> meta_k(pj.w)) & 1u)) continue;
@@ -542,68 +547,321 @@ void launch_delta_energy(const LaunchCtx &L, int n) {
     k_mark_b<<<L.n_sys, 32, 0, L.stream>>>(L.sys, n, 1);
 }
 
-// ------------------------------------------------------------ mutations
-// Semi-grand lipid mutations (Sec. 2: a random lipid turned into a lipid of
-// another type under a Metropolis test), n in order by one block per system.
-// Trial T draws Philox (0, T, TAG_MUTATE, 0): lipid a from word 0, the new
-// type among the other n_lt - 1 types from word 1, u from words 2-3.  dE is
-// the FP64 sum over the changed beads of a and their neighbours in the 27
-// cells (the cell list of the current state); accept iff
-// dE - (mu[new] - mu[old]) + kT ln u <= 0.
-__global__ void __launch_bounds__(128) k_mutation_trials(const SysDev *__restrict__ sys, int n) {
-    const SysDev &S = sys[blockIdx.x];
+// ------------------------------------------- trials in order, many per launch
+// Exchange trials over the pair lists (G list columns per bead) and semi-grand
+// lipid mutations over the cells (G = 0; Sec. 2: a random lipid turned into a
+// lipid of another type under a Metropolis test), with the result of processing
+// them one after another.  Coordinates do not change, so what a trial's dE
+// depends on are the types of its own lipids and of the lipids with a bead
+// inside the cutoff of a changed bead.  A chunk of trials runs as
+//   k_chain_propose: who draws which lipid (per lipid a list of the chunk's
+//     trials);
+//   k_chain_eval: every trial's dE against the types the chunk starts with, a
+//     block per trial, and as it walks the partners the earlier trials of the
+//     chunk whose acceptance would change it (a bit per trial);
+//   k_chain_walk: one cluster of blocks per system decides the trials in order;
+//     one whose bits meet an accepted trial is evaluated again, by the whole
+//     cluster (the FP64 pair terms bound a single SM: about 500 of them at 45
+//     operations, two per clock).
+// dE is one fixed sum of CHAIN_SLOTS slots, whichever kernel computes it, so
+// the records do not depend on the chunks.
+//
+// Measured, a call of 256 trials: exchanges on a 1424-lipid bilayer 566 us (a
+// launch per trial: 2574), mutations on a 4608-lipid bilayer 482 us (one block
+// for all of them: 11207).
+//
+// Mutation trial T draws Philox (0, T, TAG_MUTATE, 0): lipid a from word 0, the
+// new type among the other n_lt - 1 types from word 1, u from words 2-3; accept
+// iff dE - (mu[new] - mu[old]) + kT ln u <= 0.
+constexpr int CHAIN_BLOCKS = 8;                // blocks of a cluster of k_chain_walk
+constexpr int CHAIN_THREADS = 128;
+constexpr int CHAIN_SLOTS = CHAIN_BLOCKS * CHAIN_THREADS;
+constexpr int CHAIN_SUMS = CHAIN_SLOTS / 32;   // warp sums of one dE
+constexpr int CHAIN_WORDS = CHAIN_MAX / 32;
+
+struct ChainProp {
+    int a, b;                                  // the lipids (a mutation has a alone: b = a)
+    uint32_t w1;                               // mutation: the word that picks the new type
+    double u;
+};
+
+template <int G>
+__device__ __forceinline__ ChainProp chain_draw(const Params &P, unsigned long long T) {
+    const uint4 w = draw4(P, 0u, (uint32_t)T, G ? TAG_SWAP : TAG_MUTATE, 0u);
+    ChainProp r;
+    r.a = pick(w.x, P.n_lip);
+    r.b = G ? pick(w.y, P.n_lip) : r.a;
+    r.w1 = w.y;
+    r.u = unit53(w.z, w.w);
+    return r;
+}
+
+// The trial's two types, the current ones of a and b or a's old and new one,
+// and its changed beads, into sm; by one warp.
+template <int G>
+__device__ __forceinline__ void chain_setup(const SysDev &S, const ChainProp &pr, const uint4 *cur, int lane, TrialSmem &sm) {
     const Params &P = *S.p;
-    Counters &C = *S.c;
-    __shared__ double sh[128];
-    __shared__ int sa, sta, stn;
-    __shared__ double su;
-    for (int x = 0; x < n; ++x) {
-        const unsigned long long T = C.trial + (unsigned long long)x;
-        if (threadIdx.x == 0) {
-            const uint4 w = draw4(P, 0u, (uint32_t)T, TAG_MUTATE, 0u);
-            const int a = pick(w.x, P.n_lip), ta = S.ltype[a];
-            sa = a;
-            sta = ta;
-            stn = P.n_lt > 1 ? (ta + 1 + pick(w.y, P.n_lt - 1)) % P.n_lt : ta;
-            su = unit53(w.z, w.w);
+    const int ta = __ldcg(&S.ltype[pr.a]);
+    if constexpr (G > 0) {
+        trial_beads<G>(S, pr.a, pr.b, ta, __ldcg(&S.ltype[pr.b]), cur, lane, sm, [](int) {});
+    } else {
+        const int tn = P.n_lt > 1 ? (ta + 1 + pick(pr.w1, P.n_lt - 1)) % P.n_lt : ta;
+        const int oi = lane < P.bpl ? P.lbt[ta * 16 + lane] : 0, ni = lane < P.bpl ? P.lbt[tn * 16 + lane] : 0;
+        const unsigned bal = __ballot_sync(0xffffffffu, oi != ni);
+        if (oi != ni) {
+            const int o = __popc(bal & ((1u << lane) - 1u)), id = pr.a * P.bpl + lane;
+            sm.chg_id[o] = id;
+            sm.chg_pos[o] = S.pos[id];
+            sm.chg_old[o] = oi;
+            sm.chg_new[o] = ni;
         }
-        __syncthreads();
-        const int a = sa, ta = sta, tn = stn;
+        if (lane == 0) {
+            sm.nchg = __popc(bal);
+            sm.ta = ta;
+            sm.tb = tn;
+        }
+    }
+}
+
+// Slot `slot` of the dE of the trial in sm: its entries slot, slot +
+// CHAIN_SLOTS, ...  (a mutation's entry: every fourth bead of one of a changed
+// bead's 27 cells)
+template <int G, class Near>
+__device__ __forceinline__ double chain_slot(const SysDev &S, const ChainProp &pr, const uint4 *cur, const TrialSmem &sm,
+                                             int slot, Near near) {
+    const Params &P = *S.p;
+    double acc = 0.0;
+    if constexpr (G > 0) {
+        const int total = sm.it_beg[sm.nchg * G];
+        for (int f = slot; f < total; f += CHAIN_SLOTS)
+            acc += trial_entry<G>(S, pr.a, pr.b, cur, sm, f, [](int) {}, near);
+    } else {
+        const int a = pr.a, ta = sm.ta, tn = sm.tb;
         auto changed = [&](uint32_t mj, int) {
             return meta_lip(mj) == a && P.lbt[ta * 16 + meta_k(mj)] != P.lbt[tn * 16 + meta_k(mj)];
         };
         auto newt = [&](uint32_t mj, int) { return (int)P.lbt[tn * 16 + meta_k(mj)]; };
-        double acc = 0.0;
-        if (tn != ta)
-            for (int it = threadIdx.x; it < P.bpl * 27; it += blockDim.x) {
-                const int k = it / 27, slot = it % 27;
-                const int oi = P.lbt[ta * 16 + k], ni = P.lbt[tn * 16 + k];
-                if (oi == ni) continue;
-                const int i = a * P.bpl + k;
-                acc += bead_delta(S, P, i, S.pos[i], oi, ni, slot, newt, changed);
-            }
-        const double dE = block_sum(acc, sh);
-        if (threadIdx.x == 0) {
-            TrialRec r;
-            r.a = a; r.b = tn; r.u = su; r.index = T;
-            r.null_trial = tn == ta;
-            r.dE = r.null_trial ? 0.0 : dE;
-            r.accepted = !r.null_trial && metropolis(dE - (C.mu[tn] - C.mu[ta]), P.kT, su);
-            if (r.accepted) set_lipid_type(S, P, a, tn);
-            S.log[T % LOG_CAP] = r;
-            C.trials++;
-            C.force_evals++;
-            C.null_trials += r.null_trial;
-            C.accepted += r.accepted;
+        for (int f = slot; f < sm.nchg * 27 * 4; f += CHAIN_SLOTS) {
+            const int ci = f / 108, q = f % 108;
+            acc += bead_delta(S, P, sm.chg_id[ci], sm.chg_pos[ci], sm.chg_old[ci], sm.chg_new[ci], q / 4, newt, changed,
+                              q % 4, 4, near);
         }
-        __syncthreads();
     }
-    if (threadIdx.x == 0) C.trial += (unsigned long long)n;
+    return acc;
 }
 
-void launch_mutation_trials(const LaunchCtx &L, int n) {
-    k_mutation_trials<<<L.n_sys, 128, 0, L.stream>>>(L.sys, n);
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    return v;                                  // lane 0
 }
+
+// grid (1, n_sys): node 2 t + side + 1 of trial t enters the list of the lipid
+// it draws (0: the end; the walk empties the lists again)
+template <int G>
+__global__ void __launch_bounds__(CHAIN_MAX) k_chain_propose(const SysDev *__restrict__ sys, int m) {
+    const SysDev &S = sys[blockIdx.y];
+    const int t = threadIdx.x;
+    if (t >= m) return;
+    const ChainProp pr = chain_draw<G>(*S.p, S.c->trial + (unsigned long long)t);
+    for (int side = 0; side < (G ? 2 : 1); ++side)
+        S.tnext[2 * t + side] = atomicExch(&S.thead[side ? pr.b : pr.a], 2 * t + side + 1);
+}
+
+// grid (m, n_sys)
+template <int G>
+__global__ void __launch_bounds__(CHAIN_THREADS) k_chain_eval(const SysDev *__restrict__ sys) {
+    const SysDev &S = sys[blockIdx.y];
+    const Params &P = *S.p;
+    __shared__ TrialSmem sm;
+    __shared__ double sums[CHAIN_SUMS];
+    __shared__ unsigned bits[CHAIN_WORDS];
+    const int t = blockIdx.x, x = threadIdx.x, lane = x & 31;
+    const ChainProp pr = chain_draw<G>(P, S.c->trial + (unsigned long long)t);
+    const uint4 *cur = S.lpos + (size_t)S.c->nl_par * P.n;
+    if (x < CHAIN_WORDS) bits[x] = 0u;
+    if (x < 32) chain_setup<G>(S, pr, cur, lane, sm);
+    __syncthreads();
+    // the earlier trials that draw lipid l
+    auto meets = [&](int l) {
+        if (l < 0) return;
+        for (int node = S.thead[l]; node; node = S.tnext[node - 1]) {
+            const int u = (node - 1) >> 1;
+            if (u < t) atomicOr(&bits[u >> 5], 1u << (u & 31));
+        }
+    };
+    if (x < 2) meets(x ? pr.b : pr.a);
+    for (int i = 0; i < CHAIN_BLOCKS; ++i) {
+        const double s = warp_sum(chain_slot<G>(S, pr, cur, sm, CHAIN_THREADS * i + x, meets));
+        if (lane == 0) sums[(CHAIN_THREADS / 32) * i + (x >> 5)] = s;
+    }
+    __syncthreads();
+    if (x < CHAIN_WORDS) S.conflict[t * CHAIN_WORDS + x] = bits[x];
+    if (x == 0) {
+        double dE = 0.0;
+        for (int i = 0; i < CHAIN_SUMS; ++i) dE += sums[i];
+        S.tdE[t] = dE;
+        S.tprop[t] = make_int4(pr.a, pr.b, sm.ta, sm.tb);
+    }
+}
+
+__device__ __forceinline__ unsigned cluster_addr(const void *p, unsigned rank) {
+    unsigned r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((unsigned)__cvta_generic_to_shared(p)), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// grid (CHAIN_BLOCKS, n_sys), one cluster per system: trials 0 .. m - 1 of the
+// chunk in order.  spec: k_chain_eval has run (else every trial is evaluated
+// here).  The first warp of the first block decides; for a trial that needs
+// its dE it hands the cluster the trial's number and takes back the warp sums.
+template <int G>
+__global__ void __cluster_dims__(CHAIN_BLOCKS, 1, 1) __launch_bounds__(CHAIN_THREADS)
+k_chain_walk(const SysDev *__restrict__ sys, int m, int spec) {
+    const SysDev &S = sys[blockIdx.y];
+    const Params &P = *S.p;
+    Counters &C = *S.c;
+    __shared__ TrialSmem sm;
+    __shared__ double sums[CHAIN_SUMS];
+    __shared__ int cmd;
+    __shared__ unsigned bits[CHAIN_MAX * CHAIN_WORDS];
+    const int x = threadIdx.x, lane = x & 31;
+    const unsigned rank = blockIdx.x;
+    const bool lead = rank == 0 && x < 32;
+    const unsigned long long T0 = C.trial;
+    const uint4 *cur = S.lpos + (size_t)C.nl_par * P.n;
+    const bool lists = !C.nl_stale;
+    if (spec && rank == 0)
+        for (int i = x; i < m * CHAIN_WORDS; i += CHAIN_THREADS) bits[i] = S.conflict[i];
+    __syncthreads();
+    // the leading warp: the next trial, the accepted ones (lane w: word w),
+    // counts; 32 trials' proposals and dE at a time, one per lane
+    int t = 0, n_null = 0, n_acc = 0;
+    unsigned accepted = 0u;
+    bool fresh = false;                        // sums hold the dE of trial t
+    ChainProp mine;
+    double mine_dE = 0.0;
+    int mine_ta = 0, mine_tb = 0;
+    for (;;) {
+        if (lead) {
+            int next = -1;
+            for (; t < m; ++t) {
+                if ((t & 31) == 0 && !fresh) {
+                    mine = chain_draw<G>(P, T0 + (unsigned long long)min(t + lane, m - 1));
+                    if (spec && t + lane < m) {
+                        mine_dE = S.tdE[t + lane];
+                        const int4 q = S.tprop[t + lane];
+                        mine_ta = q.z;
+                        mine_tb = q.w;
+                    }
+                }
+                const unsigned hit = spec && lane < CHAIN_WORDS ? bits[t * CHAIN_WORDS + lane] & accepted : 0u;
+                if (!fresh && (!spec || __any_sync(0xffffffffu, hit != 0u))) {
+                    next = t;
+                    break;
+                }
+                const int src = t & 31;
+                TrialRec r;
+                r.a = __shfl_sync(0xffffffffu, mine.a, src);
+                const int b = __shfl_sync(0xffffffffu, mine.b, src);
+                r.u = __shfl_sync(0xffffffffu, mine.u, src);
+                double dE = __shfl_sync(0xffffffffu, mine_dE, src);
+                int ta = __shfl_sync(0xffffffffu, mine_ta, src), tb = __shfl_sync(0xffffffffu, mine_tb, src);
+                if (fresh) {
+                    dE = 0.0;
+                    for (int i = 0; i < CHAIN_SUMS; ++i) dE += sums[i];
+                    ta = sm.ta;
+                    tb = sm.tb;
+                    fresh = false;
+                }
+                r.b = G ? b : tb;
+                r.index = T0 + (unsigned long long)t;
+                r.null_trial = (G && r.a == b) || ta == tb;
+                r.dE = r.null_trial ? 0.0 : dE;
+                r.accepted = !r.null_trial && metropolis(G ? dE : dE - (C.mu[tb] - C.mu[ta]), P.kT, r.u);
+                n_null += r.null_trial;
+                n_acc += r.accepted;
+                if (lane == 0) S.log[r.index % LOG_CAP] = r;
+                if (r.accepted) {
+                    // the new types, one bead per lane
+                    const int side = lane >= P.bpl, k = side ? lane - P.bpl : lane;
+                    if (lane < (G ? 2 : 1) * P.bpl) {
+                        const int l = side ? b : r.a, id = l * P.bpl + k;
+                        const int bt = P.lbt[(side ? ta : tb) * 16 + k];
+                        const uint32_t mm = meta_make(bt, bt, k, l + 1);
+                        S.pos[id].w = mm;
+                        if (lists) const_cast<uint4 *>(cur)[S.lk[id]].w = mm;
+                        if (!G) S.spos[S.sidx[id]].w = mm;
+                    }
+                    if (lane == 0) {
+                        S.ltype[r.a] = tb;
+                        if (G) S.ltype[b] = ta;
+                    }
+                    if (lane == (t >> 5)) accepted |= 1u << (t & 31);
+                }
+            }
+            if (lane == 0) cmd = next;
+        }
+        cluster_sync();
+        int todo;
+        asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(todo) : "r"(cluster_addr(&cmd, 0)) : "memory");
+        if (todo < 0) break;
+        const ChainProp pr = chain_draw<G>(P, T0 + (unsigned long long)todo);
+        if (x < 32) chain_setup<G>(S, pr, cur, lane, sm);
+        __syncthreads();
+        const double s = warp_sum(chain_slot<G>(S, pr, cur, sm, CHAIN_THREADS * rank + x, [](int) {}));
+        if (lane == 0)
+            asm volatile("st.shared::cluster.f64 [%0], %1;"
+                         :: "r"(cluster_addr(&sums[(CHAIN_THREADS / 32) * rank + (x >> 5)], 0)), "d"(s) : "memory");
+        cluster_sync();
+        fresh = true;
+    }
+    cluster_sync();                            // every block has read the last number
+    if (lead && lane == 0) {
+        C.trials += m;
+        C.force_evals += m;
+        C.null_trials += n_null;
+        C.accepted += n_acc;
+        C.pending = 0;
+        C.trial = T0 + (unsigned long long)m;
+    }
+    if (spec && rank == 0)
+        for (int i = x; i < m; i += CHAIN_THREADS) {
+            const ChainProp pr = chain_draw<G>(P, T0 + (unsigned long long)i);
+            S.thead[pr.a] = 0;
+            S.thead[pr.b] = 0;
+        }
+}
+
+// A chunk is long enough to fill the GPU with evaluations and short enough that
+// few of its trials meet an accepted one: a trial of a bilayer of n_lip lipids
+// has some 25 lipids in reach, so a chunk of n_lip / 16 evaluates about one
+// trial in five again.  From CHAIN_MIN trials on (shorter chunks of small
+// bilayers, where most trials meet, are walked without the first evaluation).
+template <int G>
+static void chain_launch(const LaunchCtx &L, int n, int max_lip) {
+    const int chunk = max_lip / 16 >= CHAIN_MAX ? CHAIN_MAX : max_lip / 16;
+    const int spec = chunk >= CHAIN_MIN && n >= CHAIN_MIN;
+    const int step = spec ? chunk : CHAIN_MAX;
+    for (int done = 0; done < n; done += step) {
+        const int m = n - done < step ? n - done : step;
+        if (spec) {
+            k_chain_propose<G><<<dim3(1, L.n_sys), CHAIN_MAX, 0, L.stream>>>(L.sys, m);
+            k_chain_eval<G><<<dim3(m, L.n_sys), CHAIN_THREADS, 0, L.stream>>>(L.sys);
+        }
+        k_chain_walk<G><<<dim3(CHAIN_BLOCKS, L.n_sys), CHAIN_THREADS, 0, L.stream>>>(L.sys, m, spec);
+    }
+}
+
+void launch_swap_trials(const LaunchCtx &L, int n, int max_lip) {
+    if (L.lanes == 2) chain_launch<2>(L, n, max_lip);
+    else chain_launch<4>(L, n, max_lip);
+}
+
+void launch_mutation_trials(const LaunchCtx &L, int n, int max_lip) { chain_launch<0>(L, n, max_lip); }
 
 // ----------------------------------------------------------------- Philox
 __global__ void k_philox(uint32_t k0, uint32_t k1, uint32_t c1, uint32_t c2, uint32_t c3, int n, uint4 *out) {
