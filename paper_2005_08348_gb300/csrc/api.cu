@@ -997,7 +997,7 @@ mdas_status mdas_forces(mdas_system *s, double *f_out, double *u_out) {
     if (f_out) {
         mdas_status st = build_cells(s, b);
         if (st != MDAS_OK) return st;
-        launch_pair(L, false, false, s->precision == 1);
+        launch_pair(L, s->precision == 1);
         launch_total_force(L, s->fout, 0);
         CK(cudaMemcpyAsync(f_out, s->fout, 24ull * s->n, cudaMemcpyDeviceToHost, s->stream));
     }
@@ -1018,8 +1018,7 @@ mdas_status mdas_energy(mdas_system *s, mdas_energy_terms *out) {
     LaunchCtx L = b.ctx();
     mdas_status st0 = build_cells(s, b);
     if (st0 != MDAS_OK) return st0;
-    launch_pair(L, false, true, true);
-    launch_energy_reduce(L);
+    launch_energy(L);
     double r[8];
     CK(cudaMemcpyAsync(r, s->hs.result, sizeof(r), cudaMemcpyDeviceToHost, s->stream));
     CK(cudaStreamSynchronize(s->stream));

@@ -280,7 +280,7 @@ void launch_pcouple(const LaunchCtx &L) {
 // The bonded force of each i-bead (computed by the cell-list finish) joins the
 // stream partials, and the total force is stored in fixed point.
 
-template <typename Real, bool LAM, bool ENERGY>
+template <typename Real>
 __global__ void __launch_bounds__(PAIR_THREADS, 8) k_pair(const SysDev *__restrict__ sys, const int2 *__restrict__ bmap) {
     using V4 = typename Vec4<Real>::T;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -305,7 +305,6 @@ __global__ void __launch_bounds__(PAIR_THREADS, 8) k_pair(const SysDev *__restri
     __shared__ int wcnt[NW];
     __shared__ Real bx[3][PAIR_THREADS];
     __shared__ Real blo[3], bhi[3];
-    __shared__ double ered[3][PAIR_THREADS];
     __shared__ __align__(16) V4 sbf[PAIR_THREADS];       // bonded force of the chunk's i-beads
     __shared__ int sid[PAIR_THREADS];                    // their ids
 
@@ -349,10 +348,8 @@ __global__ void __launch_bounds__(PAIR_THREADS, 8) k_pair(const SysDev *__restri
     const Real rc2 = F32 ? (Real)P.rc2f : (Real)P.rc2;
     const Real rc2lo = F32 ? (Real)P.rc2f_lo : (Real)P.rc2;
     const Real krf2 = F32 ? (Real)P.krf2f : (Real)(2.0 * P.krf);
-    const Real lam = LAM ? (Real)S.c->lambda : (Real)0;
     const float qh0 = P.qsh[0], qh1 = P.qsh[1], qh2 = P.qsh[2];
     const float ql0 = P.qsl[0], ql1 = P.qsl[1], ql2 = P.qsl[2];
-    double elj = 0.0, erf = 0.0, epairs = 0.0;
 
     for (int ib = 0; ib < ni; ib += IW) {
         const int i = ib + il;
@@ -372,7 +369,7 @@ __global__ void __launch_bounds__(PAIR_THREADS, 8) k_pair(const SysDev *__restri
         if (js == 0) { bx[0][il] = pi.x; bx[1][il] = pi.y; bx[2][il] = pi.z; }
         if (!valid) pi.x = (Real)1e30;            // an idle lane never finds a partner
         const uint32_t mi = vi.w;
-        const int tai = meta_ta(mi), tbi = meta_tb(mi), ki = meta_k(mi);
+        const int tai = meta_ta(mi), ki = meta_k(mi);
         const uint32_t lipi = mi >> 12;
         const uint32_t emask = P.excl[ki];
         Real ax = 0, ay = 0, az = 0;
@@ -413,13 +410,7 @@ __global__ void __launch_bounds__(PAIR_THREADS, 8) k_pair(const SysDev *__restri
             }
             if (!keep) return;
             const int ta = tai * 16 + meta_ta(mj);
-            Real f12 = tf12[ta], f6 = tf6[ta], qq = tqq[ta];
-            if (LAM) {
-                const int tb = tbi * 16 + meta_tb(mj);
-                f12 = ((Real)1 - lam) * f12 + lam * tf12[tb];
-                f6 = ((Real)1 - lam) * f6 + lam * tf6[tb];
-                qq = ((Real)1 - lam) * qq + lam * tqq[tb];
-            }
+            const Real f12 = tf12[ta], f6 = tf6[ta], qq = tqq[ta];
             Real rinv, r2inv, r6inv;
             if (F32) {
                 const float r2i = __frcp_rn((float)r2);
@@ -435,23 +426,6 @@ __global__ void __launch_bounds__(PAIR_THREADS, 8) k_pair(const SysDev *__restri
             }
             const Real fs = (f12 * r6inv - f6) * r6inv * r2inv + qq * (rinv * r2inv - krf2);
             ax += fs * dx; ay += fs * dy; az += fs * dz;
-            if (ENERGY) {
-                const int ia = tai * 16 + meta_ta(mj);
-                double c12 = P.c12[ia], c6 = P.c6[ia], qd = P.qq[ia], sh = P.ush[ia];
-                if (LAM) {
-                    const int ibb = tbi * 16 + meta_tb(mj);
-                    const double l = (double)lam;
-                    c12 = (1 - l) * c12 + l * P.c12[ibb];
-                    c6 = (1 - l) * c6 + l * P.c6[ibb];
-                    qd = (1 - l) * qd + l * P.qq[ibb];
-                    sh = (1 - l) * sh + l * P.ush[ibb];
-                }
-                const double ri = (double)rinv, r2d = (double)r2;
-                const double r6 = ri * ri * ri * ri * ri * ri;
-                elj += 0.5 * (c12 * r6 * r6 - c6 * r6 - sh);
-                erf += 0.5 * qd * (ri + P.krf * r2d - P.crf);
-                epairs += 0.5;
-            }
         };
         // cull the staged list [0, mc) into private queues, then evaluate them
         auto process = [&](int mc) {
@@ -546,20 +520,6 @@ __global__ void __launch_bounds__(PAIR_THREADS, 8) k_pair(const SysDev *__restri
         }
         __syncthreads();                          // red (over q) is read before the next chunk
     }
-    if (ENERGY) {
-        __syncthreads();
-        ered[0][t] = elj; ered[1][t] = erf; ered[2][t] = epairs;
-        __syncthreads();
-        for (int w = PAIR_THREADS / 2; w > 0; w >>= 1) {
-            if (t < w) { ered[0][t] += ered[0][t + w]; ered[1][t] += ered[1][t + w]; ered[2][t] += ered[2][t + w]; }
-            __syncthreads();
-        }
-        if (t == 0) {
-            S.epart[4 * c + 0] = ered[0][0];
-            S.epart[4 * c + 1] = ered[1][0];
-            S.epart[4 * c + 2] = ered[2][0];
-        }
-    }
 }
 
 template <typename Real>
@@ -569,40 +529,29 @@ static size_t pair_smem() {
            sizeof(uint16_t) * QCAP * PAIR_THREADS;
 }
 
-template <typename Real, bool LAM, bool ENERGY>
+template <typename Real>
 static void pair_launch(const LaunchCtx &L) {
-    k_pair<Real, LAM, ENERGY><<<L.cells->n, PAIR_THREADS, pair_smem<Real>(), L.stream>>>(L.sys, L.cells->d);
+    k_pair<Real><<<L.cells->n, PAIR_THREADS, pair_smem<Real>(), L.stream>>>(L.sys, L.cells->d);
 }
 
-template <typename Real, bool LAM, bool ENERGY>
+template <typename Real>
 static cudaError_t pair_attr() {
-    return cudaFuncSetAttribute(k_pair<Real, LAM, ENERGY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)pair_smem<Real>());
+    return cudaFuncSetAttribute(k_pair<Real>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pair_smem<Real>());
 }
 
 // once per process, before any capture: shared-memory limits of the pair kernels
 cudaError_t setup_kernels() {
     static cudaError_t done = cudaErrorNotReady;
     if (done != cudaErrorNotReady) return done;
-    cudaError_t e = pair_attr<float, false, false>();
-    if (e == cudaSuccess) e = pair_attr<float, true, false>();
-    if (e == cudaSuccess) e = pair_attr<double, false, false>();
-    if (e == cudaSuccess) e = pair_attr<double, true, false>();
-    if (e == cudaSuccess) e = pair_attr<double, false, true>();
-    if (e == cudaSuccess) e = pair_attr<double, true, true>();
+    cudaError_t e = pair_attr<float>();
+    if (e == cudaSuccess) e = pair_attr<double>();
     done = e;
     return e;
 }
 
-// forces only (fixed point, pair + bonded) or energies
-void launch_pair(const LaunchCtx &L, bool lambda, bool energy, bool fp64) {
-    if (energy) {
-        if (lambda) pair_launch<double, true, true>(L); else pair_launch<double, false, true>(L);
-    } else if (fp64) {
-        if (lambda) pair_launch<double, true, false>(L); else pair_launch<double, false, false>(L);
-    } else {
-        if (lambda) pair_launch<float, true, false>(L); else pair_launch<float, false, false>(L);
-    }
+// forces (fixed point, pair + bonded)
+void launch_pair(const LaunchCtx &L, bool fp64) {
+    if (fp64) pair_launch<double>(L); else pair_launch<float>(L);
 }
 
 // total force of one system (fixed point) as double, for the host
@@ -673,6 +622,126 @@ __global__ void __launch_bounds__(BEAD_BLOCK) k_bonded_energy(const SysDev *__re
     if (threadIdx.x < 3) S.bpart[3 * (bm.y / BEAD_BLOCK) + threadIdx.x] = part[threadIdx.x][0];
 }
 
+// FP64 Lennard-Jones and reaction-field energy and the pairs inside rc, per
+// cell into epart; a warp per cell.  Every unordered pair counts once: the
+// candidates are the later beads of the cell itself and those of the 13
+// neighbour cells ahead of it.  The warp takes 32 candidates at a time, one per
+// lane, and tests them against each of the cell's beads in FP32 (from exact
+// integer offsets; a bound that no pair inside rc fails); the pairs that pass
+// wait in a ring until 32 are there, and then each lane takes one through FP64.
+//
+// The FP64 pipe bounds it (two operations per clock and SM): each pair goes
+// through it once, at about 27 operations with 1/r from a float seed and two
+// Newton steps, the last in the residual form (within an ulp), where the force
+// kernel's pass took every pair twice with a square root, a division and the
+// forces (a call for forces and energies, 1152 lipids: 654 to 334 us).
+constexpr int ENERGY_WARPS = 4;
+__global__ void __launch_bounds__(32 * ENERGY_WARPS) k_cell_energy(const SysDev *__restrict__ sys,
+                                                                   const int2 *__restrict__ bmap, int n_items) {
+    constexpr unsigned FULL = 0xffffffffu;
+    __shared__ int4 ring[ENERGY_WARPS][64];       // integer separation, type pair
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int item = blockIdx.x * ENERGY_WARPS + w;
+    if (item >= n_items) return;
+    const int2 bm = bmap[item];
+    const SysDev &S = sys[bm.x];
+    const Params &P = *S.p;
+    const int c = bm.y;
+    const int nx = P.nc[0], ny = P.nc[1], nz = P.nc[2];
+    const int cz = c / (nx * ny), cxy = c - cz * nx * ny, cy = cxy / nx, cx = cxy - cy * nx;
+    // lane q < 14: first bead and count of the cell itself (q = 0) and of the
+    // neighbours ahead (offsets 13 + q of the 27), and the candidates before
+    int first = 0, cnt = 0;
+    if (lane < 14) {
+        const int o = 13 + lane, dz = o / 9 - 1, dy = (o / 3) % 3 - 1, dx = o % 3 - 1;
+        int x = cx + dx, y = cy + dy, z = cz + dz;
+        x += x < 0 ? nx : (x >= nx ? -nx : 0);
+        y += y < 0 ? ny : (y >= ny ? -ny : 0);
+        z += z < 0 ? nz : (z >= nz ? -nz : 0);
+        const int cj = (z * ny + y) * nx + x;
+        first = cj * P.capc;
+        cnt = S.cell_n[cj];
+    }
+    int off = cnt;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int x = __shfl_up_sync(FULL, off, d);
+        if (lane >= d) off += x;
+    }
+    const int M = __shfl_sync(FULL, off, 31);
+    off -= cnt;                                   // lanes 14 .. 31: M
+    const int first_of = first - off;             // place of candidate t of cell q: t + first_of
+    const int i0 = __shfl_sync(FULL, first, 0), ni = __shfl_sync(FULL, cnt, 0);
+    const float q0 = P.qsf[0], q1 = P.qsf[1], q2 = P.qsf[2], rc2f = P.rc2f;
+    double elj = 0.0, erf = 0.0, pairs = 0.0;
+    int head = 0, tail = 0;
+    auto evaluate = [&](int nt) {
+        if (lane < nt) {
+            const int4 e = ring[w][(head + lane) & 63];
+            const double x = (double)e.x * P.qs[0], y = (double)e.y * P.qs[1], z = (double)e.z * P.qs[2];
+            const double r2 = fma(x, x, fma(y, y, z * z));
+            if (r2 < P.rc2) {
+                double ri = (double)rsqrtf((float)r2);
+                ri = ri * fma(-0.5 * r2, ri * ri, 1.5);
+                ri = fma(0.5 * ri, fma(-(r2 * ri), ri, 1.0), ri);
+                const double r2i = ri * ri, r6 = r2i * r2i * r2i;
+                elj += fma(fma(P.c12[e.w], r6, -P.c6[e.w]), r6, -P.ush[e.w]);
+                erf = fma(P.qq[e.w], fma(P.krf, r2, ri - P.crf), erf);
+                pairs += 1.0;
+            }
+        }
+        head += nt;
+        __syncwarp();
+    };
+    for (int ib = 0; ib < ni; ib += 32) {
+        // lane b holds bead ib + b of the cell
+        const int nb = min(32, ni - ib);
+        const uint4 mine = S.spos[i0 + ib + (lane < nb ? lane : 0)];
+        for (int tb = 0; tb < M; tb += 32) {
+            const int t = tb + lane;
+            int q = 0;                            // the last cell with off[q] <= t
+#pragma unroll
+            for (int d = 8; d > 0; d >>= 1) {
+                const int o = __shfl_sync(FULL, off, q + d);
+                if (o <= t) q += d;
+            }
+            const int pj = __shfl_sync(FULL, first_of, q) + t;
+            const bool v = t < M;
+            const uint4 vj = v ? S.spos[pj] : make_uint4(0u, 0u, 0u, 0u);
+            for (int b = 0; b < nb; ++b) {
+                const uint32_t xi = __shfl_sync(FULL, mine.x, b), yi = __shfl_sync(FULL, mine.y, b),
+                               zi = __shfl_sync(FULL, mine.z, b), mi = __shfl_sync(FULL, mine.w, b);
+                const int ix = (int)(xi - vj.x), iy = (int)(yi - vj.y), iz = (int)(zi - vj.z);
+                const float fx = (float)ix * q0, fy = (float)iy * q1, fz = (float)iz * q2;
+                const float r2 = fx * fx + fy * fy + fz * fz;
+                // in the cell itself the later beads only; a bonded pair does not count
+                const bool excl = (mi >> 12) != 0u && ((mi ^ vj.w) >> 12) == 0u && ((P.excl[meta_k(mi)] >> meta_k(vj.w)) & 1u);
+                const bool in = v && r2 < rc2f && r2 > 0.f && !excl && (t >= ni || t > ib + b);
+                const unsigned bal = __ballot_sync(FULL, in);
+                if (in)
+                    ring[w][(tail + __popc(bal & ((1u << lane) - 1u))) & 63] =
+                        make_int4(ix, iy, iz, meta_ta(mi) * 16 + meta_ta(vj.w));
+                tail += __popc(bal);
+                __syncwarp();
+                if (tail - head >= 32) evaluate(32);
+            }
+        }
+    }
+    if (tail != head) evaluate(tail - head);
+    // fixed-order sums
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        elj += __shfl_xor_sync(FULL, elj, o);
+        erf += __shfl_xor_sync(FULL, erf, o);
+        pairs += __shfl_xor_sync(FULL, pairs, o);
+    }
+    if (lane == 0) {
+        S.epart[4 * c + 0] = elj;
+        S.epart[4 * c + 1] = erf;
+        S.epart[4 * c + 2] = pairs;
+    }
+}
+
 // fixed-order tree sums: result[0..5] = lj, rf, bond, angle, kinetic, pairs
 __global__ void __launch_bounds__(256) k_energy_reduce(const SysDev *__restrict__ sys, const int2 *__restrict__ bmap) {
     const SysDev &S = sys[bmap[blockIdx.x].x];
@@ -694,7 +763,10 @@ __global__ void __launch_bounds__(256) k_energy_reduce(const SysDev *__restrict_
     if (t < 6) S.result[t] = sh[t][0];
 }
 
-void launch_energy_reduce(const LaunchCtx &L) {
+// FP64 energy terms of every system (a current cell list)
+void launch_energy(const LaunchCtx &L) {
+    k_cell_energy<<<(L.cells->n + ENERGY_WARPS - 1) / ENERGY_WARPS, 32 * ENERGY_WARPS, 0, L.stream>>>(L.sys, L.cells->d,
+                                                                                                      L.cells->n);
     k_bonded_energy<<<L.beads->n, BEAD_BLOCK, 0, L.stream>>>(L.sys, L.beads->d);
     k_energy_reduce<<<L.syss->n, 256, 0, L.stream>>>(L.sys, L.syss->d);
 }

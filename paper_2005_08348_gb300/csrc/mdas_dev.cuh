@@ -368,7 +368,7 @@ int md_run_groups(int precision, int mode, int lanes);
 cudaError_t setup_kernels();
 void launch_cells(const LaunchCtx &L);
 void launch_thermo_draws(const LaunchCtx &L, int n_steps);
-void launch_pair(const LaunchCtx &L, bool lambda, bool energy, bool fp64);
+void launch_pair(const LaunchCtx &L, bool fp64);
 void launch_total_force(const LaunchCtx &L, double *out, int sys_index);
 // pair-list MD: thermostat factor of the coming step (kernels.cu); list build
 // (its kernels return at once for systems whose list is valid), one step of
@@ -391,7 +391,7 @@ cudaError_t launch_barrier_stall(void *sync, cudaStream_t stream);
 // step counter is a multiple of its nstpcouple (kernels.cu)
 void launch_pcouple(const LaunchCtx &L);
 void launch_trial_nl(const LaunchCtx &L);
-void launch_energy_reduce(const LaunchCtx &L);
+void launch_energy(const LaunchCtx &L);
 
 // swap.cu launchers
 void launch_swap_propose(const LaunchCtx &L, int n_trials);
