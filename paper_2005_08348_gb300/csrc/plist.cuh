@@ -702,7 +702,13 @@ __device__ __forceinline__ void nl_step_item(int k0, int par, int *viol, const G
             r2inv = (Real)r2i;
             rinv = (Real)ri;
         } else {
-            rinv = (Real)(1.0 / sqrt((double)e.r2));
+            // 1/r from a float seed and two Newton steps, the second in the
+            // residual form (an error within an ulp, as the square root and the
+            // division had, at a fifth of their operations)
+            double ri = (double)rsqrtf((float)e.r2);
+            ri = ri * fma(-0.5 * (double)e.r2, ri * ri, 1.5);
+            ri = fma(0.5 * ri, fma(-((double)e.r2 * ri), ri, 1.0), ri);
+            rinv = (Real)ri;
             r2inv = rinv * rinv;
             r6inv = r2inv * r2inv * r2inv;
         }
@@ -737,6 +743,47 @@ __device__ __forceinline__ void nl_step_item(int k0, int par, int *viol, const G
     unsigned long long aw = 0;
     for (int pass = 0;; ++pass) {
         const int4 *nxt = lst + rs;
+        if constexpr (!F32) {
+            // FP64: the pipe (two operations per clock and SM) bounds the step,
+            // so an entry goes through it only when an FP32 test of the exact
+            // offsets (a bound that no pair inside rc fails) has let it pass.
+            // 44% do; 64 rows at a time, a lane keeps them as bits and then
+            // takes them in the order of the rows, so that the warp's lanes do
+            // so together (the bead itself, which pads the last group, fails).
+            auto passes = [&](uint4 pj) {
+                const float fx = (float)(int)(pi.x - pj.x) * qs0, fy = (float)(int)(pi.y - pj.y) * qs1,
+                            fz = (float)(int)(pi.z - pj.z) * qs2;
+                const float r2 = fmaf(fx, fx, fmaf(fy, fy, fz * fz));
+                return r2 < P.rc2f && r2 > 0.f;
+            };
+            if (4 < rows) j = rows4(nxt);
+            for (int m0 = 0; m0 < rows; m0 += 64) {
+                unsigned long long hits = 0;
+                for (int m = m0; m < min(rows, m0 + 64); m += 4) {
+                    unsigned h = (unsigned)passes(q0) | (unsigned)passes(q1) << 1;
+                    q0 = cur[j.x]; q1 = cur[j.y];
+                    h |= (unsigned)passes(q2) << 2 | (unsigned)passes(q3) << 3;
+                    q2 = cur[j.z]; q3 = cur[j.w];
+                    nxt += rs;
+                    if (m + 8 < rows) j = rows4(nxt);
+                    hits |= (unsigned long long)h << (m - m0);
+                }
+                auto entry = [&]() {                   // the list index of the first row left
+                    const int r = m0 + __ffsll((long long)hits) - 1;
+                    return MDAS_IDX(C, reinterpret_cast<const int *>(lst + (size_t)(r >> 2) * rs)[r & 3], n);
+                };
+                uint4 p = pi;
+                if (hits) p = cur[entry()];
+                while (hits) {
+                    hits &= hits - 1;
+                    int jn = 0;
+                    if (hits) jn = entry();
+                    const Sep e = cull(p);
+                    if (hits) p = cur[jn];
+                    add(e);
+                }
+            }
+        } else {
         if (4 < rows) j = rows4(nxt);
         for (int m = 0; m < rows; m += 4) {
             {
@@ -759,6 +806,7 @@ __device__ __forceinline__ void nl_step_item(int k0, int par, int *viol, const G
                 if (m + 8 < rows) j = rows4(nxt);
                 add(a); add(b);
             }
+        }
         }
         // this lane's share of the bead's bonded terms (partners staged by all
         // lanes of the bead: wait for the copies, then the warp barrier); the
