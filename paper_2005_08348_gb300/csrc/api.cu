@@ -209,7 +209,7 @@ void destroy_batch(Batch *b) {
 }
 
 // block maps of a batch: per system its bead blocks, cells, cell groups of the
-// cell-list finish (plus the thermostat block), step-kernel blocks and
+// cell-list finish, step-kernel blocks and
 // list-build place items (four cells each)
 struct Maps {
     std::vector<int2> beads, cells, sortcells, syss, nlbeads, lsort;
@@ -221,7 +221,6 @@ void Maps::add(int k, const mdas_system *x) {
     for (int i = 0; i < x->n; i += BEAD_BLOCK) beads.push_back(make_int2(k, i));
     for (int c = 0; c < x->hp.n_cells; ++c) cells.push_back(make_int2(k, c));
     for (int c = 0; c < x->hp.n_cells; c += CELLS_PER_SORT_BLOCK) sortcells.push_back(make_int2(k, c));
-    sortcells.push_back(make_int2(k, -1));   // the system's thermostat block
     syss.push_back(make_int2(k, 0));
     for (int i = 0; i < x->n; i += NL_BLOCK / lanes) nlbeads.push_back(make_int2(k, i));
     for (int c = 0; c < x->hp.n_lcells; c += CELLS_PER_SORT_BLOCK) lsort.push_back(make_int2(k, c));
@@ -337,7 +336,7 @@ mdas_status build_cells(mdas_system *s, Batch &b) {
     return MDAS_OK;
 }
 
-__global__ void k_batch_status(const SysDev *__restrict__ sys, int n, int *out) {
+__device__ void batch_status_warp(const SysDev *__restrict__ sys, int n, int *out) {
     int pend = 0, err = 0;
     for (int k = threadIdx.x; k < n; k += blockDim.x) { pend += sys[k].c->pending; err |= sys[k].c->err; }
     for (int o = 16; o > 0; o >>= 1) {
@@ -347,8 +346,11 @@ __global__ void k_batch_status(const SysDev *__restrict__ sys, int n, int *out) 
     if (threadIdx.x == 0) { out[0] = pend; out[1] = err; }
 }
 
-mdas_status batch_status(mdas_system *s, Batch &b, int *pending, int *err) {
-    k_batch_status<<<1, 32, 0, b.stream>>>(b.dsys, (int)b.sys.size(), b.dscratch);
+__global__ void k_batch_status(const SysDev *__restrict__ sys, int n, int *out) { batch_status_warp(sys, n, out); }
+
+// summed: the batch's last kernel has left the status in dscratch
+mdas_status batch_status(mdas_system *s, Batch &b, int *pending, int *err, bool summed = false) {
+    if (!summed) k_batch_status<<<1, 32, 0, b.stream>>>(b.dsys, (int)b.sys.size(), b.dscratch);
     int h[2];
     CK(cudaMemcpyAsync(h, b.dscratch, sizeof(h), cudaMemcpyDeviceToHost, b.stream));
     CK(cudaStreamSynchronize(b.stream));
@@ -357,9 +359,9 @@ mdas_status batch_status(mdas_system *s, Batch &b, int *pending, int *err) {
     return MDAS_OK;
 }
 
-mdas_status check_err(mdas_system *s, Batch &b) {
+mdas_status check_err(mdas_system *s, Batch &b, bool summed = false) {
     int pend, err;
-    mdas_status st = batch_status(s, b, &pend, &err);
+    mdas_status st = batch_status(s, b, &pend, &err, summed);
     if (st != MDAS_OK) return st;
     if (err) {
         for (auto *x : b.sys) x->unstable = true;
@@ -407,18 +409,22 @@ struct SegTimer {
     }
 };
 
-__global__ void k_run_abort(void *sync, int nbytes, const SysDev *__restrict__ sys, int n_sys, SysBar *bars) {
-    // a persistent launch that gave up at a barrier: every system of the
-    // batch records it, and the barrier state is cleared for the next launch
+// After a persistent launch (one warp): if it gave up at a barrier, every
+// system of the batch records it, and the barrier state is cleared for the next
+// launch.  status: the batch's status too (the call's last launch), which
+// saves a kernel of its own.
+__global__ void k_run_end(void *sync, int nbytes, const SysDev *__restrict__ sys, int n_sys, SysBar *bars, int *status) {
     const int *w = (const int *)sync;
     const int ab = w[2];
-    if (ab == 0) return;
-    for (int q = threadIdx.x; q < n_sys; q += blockDim.x) {
-        atomicOr(&sys[q].c->err, ab);
-        if (bars) bars[q].count = bars[q].base = 0u;
+    if (ab != 0) {
+        for (int q = threadIdx.x; q < n_sys; q += blockDim.x) {
+            atomicOr(&sys[q].c->err, ab);
+            if (bars) bars[q].count = bars[q].base = 0u;
+        }
+        __syncwarp();
+        if (threadIdx.x == 0) memset(sync, 0, nbytes);
     }
-    __syncthreads();
-    if (threadIdx.x == 0) memset(sync, 0, nbytes);
+    if (status) batch_status_warp(sys, n_sys, status);
 }
 
 // The partition of a persistent launch's groups among the systems of a
@@ -552,20 +558,23 @@ mdas_status run_md(mdas_system *s, Batch &b, long long n_steps, int swap_every, 
             }
         }
     }
+    bool summed = false;                       // the last launch has left the batch's status
     for (long long k0 = 0, n = 0; k0 < n_steps; k0 += n) {
         n = std::min(seg, n_steps - k0);
         if (pc_nst > 0) n = std::min(n, pc_nst - (pc_phase + k0) % pc_nst);
-        launch_thermo_draws(L, (int)std::min<long long>(n + 1, MAX_DRAW_STEPS));
-        launch_thermostat(L);
-        launches += 2;
+        launch_thermo(L, (int)std::min<long long>(n + 1, MAX_DRAW_STEPS));
+        launches += 1;
         if (persistent) {
             CK(tm.begin(b.stream, n));
             CK(launch_md_run(L, lambda, (int)n, swap_every, trial ? (int)(k0 % swap_every) : 0, lam_M,
                              (int)(lam_base + k0), dlam, b.rsync));
             CK(tm.end(b.stream));
-            k_run_abort<<<1, 32, 0, b.stream>>>(b.rsync, (int)md_run_sync_bytes(), b.dsys, (int)b.sys.size(),
-                                                 L.part ? (SysBar *)((char *)L.part + part_layout((int)b.sys.size(),
-                                                          L.part_groups).bars) : nullptr);
+            // (a box update after it can raise an error of its own)
+            summed = pc_nst == 0 && k0 + n >= n_steps;
+            k_run_end<<<1, 32, 0, b.stream>>>(b.rsync, (int)md_run_sync_bytes(), b.dsys, (int)b.sys.size(),
+                                              L.part ? (SysBar *)((char *)L.part + part_layout((int)b.sys.size(),
+                                                       L.part_groups).bars) : nullptr,
+                                              summed ? b.dscratch : nullptr);
             launches += 1;
             if (pc_nst > 0) { launch_pcouple(L); ++launches; }
             continue;
@@ -600,7 +609,7 @@ mdas_status run_md(mdas_system *s, Batch &b, long long n_steps, int swap_every, 
     for (auto *x : b.sys) x->kernel_launches += launches;
     CK(cudaGetLastError());
     CK(tm.collect(b));
-    return check ? check_err(s, b) : MDAS_OK;
+    return check ? check_err(s, b, summed) : MDAS_OK;
 }
 
 // n exchange trials per system of a batch with sequential semantics.
@@ -1374,7 +1383,7 @@ mdas_status mdas_wait_timeout_probe(mdas_system *s) {
     if (!s) return fail(nullptr, MDAS_ERR_INVALID_ARG, "wait_timeout_probe: NULL system");
     Batch &b = *s->solo;
     CK(launch_barrier_stall(b.rsync, b.stream));
-    k_run_abort<<<1, 32, 0, b.stream>>>(b.rsync, (int)md_run_sync_bytes(), b.dsys, (int)b.sys.size(), nullptr);
+    k_run_end<<<1, 32, 0, b.stream>>>(b.rsync, (int)md_run_sync_bytes(), b.dsys, (int)b.sys.size(), nullptr, nullptr);
     CK(cudaGetLastError());
     return check_err(s, b);
 }

@@ -94,23 +94,15 @@ __device__ void finish_cell(const SysDev &S, const Params &P, int c, int lane) {
 }
 
 template <typename Real>
-__device__ void thermostat_block(const SysDev &S, const Params &P);
-
-template <typename Real>
 __global__ void k_cell_finish(const SysDev *__restrict__ sys, const int2 *__restrict__ bmap) {
     const int2 bm = bmap[blockIdx.x];
     const SysDev &S = sys[bm.x];
     const Params &P = *S.p;
-    if (bm.y < 0) {                              // the system's thermostat block
-        thermostat_block<Real>(S, P);
-        return;
-    }
     const int c = bm.y + (threadIdx.x >> 5);
     if (c < P.n_cells) finish_cell<Real>(S, P, c, threadIdx.x & 31);
 }
 
-// count every bead into its cell, then order the cells (the finish grid
-// carries one extra block per system that sets the thermostat factor)
+// count every bead into its cell, then order the cells
 void launch_cells(const LaunchCtx &L) {
     k_cell_count<<<L.beads->n, BEAD_BLOCK, 0, L.stream>>>(L.sys, L.beads->d);
     if (L.precision == 1)
@@ -120,43 +112,27 @@ void launch_cells(const LaunchCtx &L) {
 }
 
 // ------------------------------------------------------------ thermostat
-// grid (ceil(2 n / 64), n_sys): variates for the next n MD steps of the
-// current counter domain (plain MD or alchemical trajectory)
-__global__ void k_thermo_draws(const SysDev *__restrict__ sys, int n) {
-    const SysDev &S = sys[blockIdx.y];
-    const Params &P = *S.p;
-    Counters &C = *S.c;
-    const int in_at = C.in_at;
-    const unsigned long long base = in_at ? C.at_step : C.step;
-    const uint32_t tag = in_at ? TAG_AT_THERMO : TAG_THERMO;
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < 2 * n && P.tau_t > 0.0) {
-        const int g = k & 1;
-        S.tdraw[k] = bussi_draws(P, P.nf[g], (uint32_t)g, (uint32_t)(base + (k >> 1)), tag);
-    }
-    if (k == 0) { C.draw_base = base; C.draw_n = P.tau_t > 0.0 ? n : 0; C.draw_tag = (int)tag; }
-}
-
-void launch_thermo_draws(const LaunchCtx &L, int n) {
-    n = n < MAX_DRAW_STEPS ? n : MAX_DRAW_STEPS;
-    dim3 g((2 * n + 63) / 64, L.n_sys);
-    k_thermo_draws<<<g, 64, 0, L.stream>>>(L.sys, n);
-}
-
 // Thermostat factor of the coming step (counter C.step, or C.at_step on the
 // alchemical trajectory): group kinetic energies as the last MD step left
 // them (ke_fresh), else straight from the velocities; fixed-order reductions
 // (thread-strided sums, a shuffle tree per warp, the warps in order by a
-// shuffle tree in warp 0).  Any block size that is a multiple of 32.
+// shuffle tree in warp 0).  Any block size that is a multiple of 32, at least
+// 64: the last warp draws the step's variates meanwhile (a lane each).
 template <typename Real>
 __device__ void thermostat_block(const SysDev &S, const Params &P) {
     using V4 = typename Vec4<Real>::T;
     Counters &C = *S.c;
     const int t = threadIdx.x, T = blockDim.x, lane = t & 31;
     __shared__ Real ws[2][32];
+    __shared__ double draw[4];
     __shared__ int fresh;
     if (t == 0) fresh = C.ke_fresh;
     __syncthreads();
+    if (t >= T - 32 && lane < 4 && P.tau_t > 0.0) {
+        const int in_at = C.in_at;
+        draw[lane] = bussi_draw(P, P.nf[lane >> 1], (uint32_t)(lane >> 1), (uint32_t)(in_at ? C.at_step : C.step),
+                                in_at ? TAG_AT_THERMO : TAG_THERMO, lane & 1);
+    }
     Real k0 = 0, k1 = 0;
     if (fresh) {
         if (t == 0) { k0 = (Real)C.ke_total[0]; k1 = (Real)C.ke_total[1]; }
@@ -185,27 +161,48 @@ __device__ void thermostat_block(const SysDev &S, const Params &P) {
             k0 += __shfl_xor_sync(0xffffffffu, k0, o);
             k1 += __shfl_xor_sync(0xffffffffu, k1, o);
         }
-        const int in_at = C.in_at;
-        const unsigned long long ctr = in_at ? C.at_step : C.step;
-        const uint32_t tag = in_at ? TAG_AT_THERMO : TAG_THERMO;
         if (lane < 2) {                         // lane g: coupling group g
-            C.alpha[lane] = alpha_for(S, P, C, lane, (double)(lane == 0 ? k0 : k1), ctr, tag);
+            C.alpha[lane] = alpha_of(P, lane, (double)(lane == 0 ? k0 : k1), make_double2(draw[2 * lane], draw[2 * lane + 1]));
             C.alpha_f[lane] = (float)C.alpha[lane];
         }
     }
 }
 
-// grid (n_sys): the thermostat factor of the coming step of every system
+// Before an MD segment of n steps: grid (blocks of variates + 1, n_sys).  The
+// last block of a system sets the factor of its first step (thermostat_block);
+// the others draw the variates of the segment, a warp of 32 each: two groups,
+// and R1 and S of a step apart.  The variates are FP64 logarithms, roots and a
+// cosine, which the FP64 pipe (two operations per clock and SM) bounds: a warp
+// per SM.  One launch, both parts beside each other, where two kernels went one
+// after the other: with the ending merged too, calls of 20 steps are 1 to 3%
+// shorter and 64 mutation trials took 332 us for 400.
 constexpr int THERMO_THREADS = 1024;
 template <typename Real>
-__global__ void __launch_bounds__(THERMO_THREADS) k_thermostat(const SysDev *__restrict__ sys) {
-    const SysDev &S = sys[blockIdx.x];
-    thermostat_block<Real>(S, *S.p);
+__global__ void __launch_bounds__(THERMO_THREADS) k_thermo(const SysDev *__restrict__ sys, int n) {
+    const SysDev &S = sys[blockIdx.y];
+    const Params &P = *S.p;
+    Counters &C = *S.c;
+    if (blockIdx.x + 1 == gridDim.x) {
+        thermostat_block<Real>(S, P);
+        return;
+    }
+    if (threadIdx.x >= 32) return;
+    const int in_at = C.in_at;
+    const unsigned long long base = in_at ? C.at_step : C.step;
+    const uint32_t tag = in_at ? TAG_AT_THERMO : TAG_THERMO;
+    const int k = blockIdx.x * 32 + threadIdx.x;   // step k / 4, group (k / 2) % 2, R1 or S
+    if (k < 4 * n && P.tau_t > 0.0) {
+        const int g = (k >> 1) & 1;
+        reinterpret_cast<double *>(S.tdraw)[k] = bussi_draw(P, P.nf[g], (uint32_t)g, (uint32_t)(base + (k >> 2)), tag, k & 1);
+    }
+    if (k == 0) { C.draw_base = base; C.draw_n = P.tau_t > 0.0 ? n : 0; C.draw_tag = (int)tag; }
 }
 
-void launch_thermostat(const LaunchCtx &L) {
-    if (L.precision == 1) k_thermostat<double><<<L.n_sys, THERMO_THREADS, 0, L.stream>>>(L.sys);
-    else k_thermostat<float><<<L.n_sys, THERMO_THREADS, 0, L.stream>>>(L.sys);
+void launch_thermo(const LaunchCtx &L, int n) {
+    n = n < MAX_DRAW_STEPS ? n : MAX_DRAW_STEPS;
+    const dim3 g((4 * n + 31) / 32 + 1, L.n_sys);
+    if (L.precision == 1) k_thermo<double><<<g, THERMO_THREADS, 0, L.stream>>>(L.sys, n);
+    else k_thermo<float><<<g, THERMO_THREADS, 0, L.stream>>>(L.sys, n);
 }
 
 // Pressure coupling after an MD segment (Sec. 3: semi-isotropic

@@ -367,16 +367,16 @@ int md_run_groups(int precision, int mode, int lanes);
 
 cudaError_t setup_kernels();
 void launch_cells(const LaunchCtx &L);
-void launch_thermo_draws(const LaunchCtx &L, int n_steps);
 void launch_pair(const LaunchCtx &L, bool fp64);
 void launch_total_force(const LaunchCtx &L, double *out, int sys_index);
-// pair-list MD: thermostat factor of the coming step (kernels.cu); list build
+// pair-list MD: the variates of the next n steps and the thermostat factor of
+// the coming one (kernels.cu); list build
 // (its kernels return at once for systems whose list is valid), one step of
 // every system (plist.cu); a whole MD segment in one cooperative launch of
 // the persistent kernel (cudaErrorCooperativeLaunchTooLarge when it cannot
 // run resident on this device), with a zeroed device RunSync of
 // md_run_sync_bytes() bytes per batch
-void launch_thermostat(const LaunchCtx &L);
+void launch_thermo(const LaunchCtx &L, int n);
 void launch_nl_build(const LaunchCtx &L);
 void launch_nl_step(const LaunchCtx &L, bool lambda);
 int md_run_blocks(int precision, int mode, int lanes);   // mode: 0 plain MD, 1 linear alchemical path,

@@ -41,13 +41,15 @@ __device__ inline double gamma_variate(const Params &P, uint32_t i0, uint32_t i1
 }
 
 // The two random variates of one Bussi et al. (2007) rescaling: R1 ~ N(0, 1)
-// from Philox call 0 and S ~ chi2(nf - 1) from calls >= 1 of counter
-// (g, ctr, tag).  They depend on the counters only, so a whole segment's
-// worth is drawn in parallel ahead of the steps.
+// (which = 0) from Philox call 0 and S ~ chi2(nf - 1) (which = 1) from calls >=
+// 1 of counter (g, ctr, tag).  They depend on the counters only, so a whole
+// segment's worth is drawn in parallel ahead of the steps.
+__device__ inline double bussi_draw(const Params &P, int nf, uint32_t g, uint32_t ctr, uint32_t tag, int which) {
+    if (which == 0) return normal_of(draw4(P, g, ctr, tag, 0));
+    return nf >= 3 ? 2.0 * gamma_variate(P, g, ctr, tag, 0.5 * (nf - 1), 1) : 0.0;
+}
 __device__ inline double2 bussi_draws(const Params &P, int nf, uint32_t g, uint32_t ctr, uint32_t tag) {
-    const double r1 = normal_of(draw4(P, g, ctr, tag, 0));
-    const double S = nf >= 3 ? 2.0 * gamma_variate(P, g, ctr, tag, 0.5 * (nf - 1), 1) : 0.0;
-    return make_double2(r1, S);
+    return make_double2(bussi_draw(P, nf, g, ctr, tag, 0), bussi_draw(P, nf, g, ctr, tag, 1));
 }
 
 // Rescaling factor: new kinetic energy (sqrt(c K) + R1 sqrt((1-c) Kt/Nf))^2 +
@@ -70,6 +72,13 @@ __device__ inline float bussi_alpha_f(const Params &P, double K, int nf, double 
     return sqrtf(knew / Kf);
 }
 
+// Factor of group g from its kinetic energy and variates, in the system's precision.
+__device__ inline double alpha_of(const Params &P, int g, double K, double2 d) {
+    if (P.tau_t <= 0.0) return 1.0;
+    return P.precision == 1 ? bussi_alpha(P, K, P.nf[g], P.ktarget[g], d)
+                            : (double)bussi_alpha_f(P, K, P.nf[g], P.ktarget[g], d);
+}
+
 // Factor of group g for the step with counter ctr of the current domain,
 // from the precomputed variates when they cover ctr.
 __device__ inline double alpha_for(const SysDev &S, const Params &P, const Counters &C, int g, double K,
@@ -80,8 +89,7 @@ __device__ inline double alpha_for(const SysDev &S, const Params &P, const Count
         d = S.tdraw[2 * (ctr - C.draw_base) + g];
     else
         d = bussi_draws(P, P.nf[g], (uint32_t)g, (uint32_t)ctr, tag);
-    return P.precision == 1 ? bussi_alpha(P, K, P.nf[g], P.ktarget[g], d)
-                            : (double)bussi_alpha_f(P, K, P.nf[g], P.ktarget[g], d);
+    return alpha_of(P, g, K, d);
 }
 
 
