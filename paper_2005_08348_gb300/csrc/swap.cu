@@ -303,54 +303,63 @@ void launch_swap_resolve(const LaunchCtx &L, int n) {
 }
 
 // ------------------------------------------------------------------ MDAS
-// Pick up to n_pairs disjoint lipid pairs of different types: candidate j
-// from Philox call (j, move, TAG_MDAS_PAIR, 0), skipped when the lipids
-// coincide, share a type, or one is already used.  Then mark the B types.
 // The pairs of an alchemical move: explicit (mode 1), drawn over all lipids
 // (mode 0, Philox (j, move, TAG_MDAS_PAIR, 0) for candidate j), or drawn
 // across the leaflets (mode 2, Philox (j, move, TAG_LEAFLET, 0); a candidate
 // is kept when a lies in leaflet 0 and b in leaflet 1 by leaf[]).  Then the
 // B types of the pairs' beads.
-__global__ void k_mdas_select(const SysDev *__restrict__ sys, int n_pairs, int max_tries, int mode,
-                              const int *__restrict__ leaf) {
+//
+// One block per system: its first warp draws 32 candidates at a time and takes
+// them in order, then every thread marks beads (one thread for all of it spent
+// its time in some 400 dependent loads, 60 us for 8 pairs; a move of 6 pairs
+// over 18 steps at 700 lipids takes 1018 us for 1053).
+constexpr int MDAS_THREADS = 128;
+static_assert(2 * MAX_PAIRS <= MDAS_THREADS, "a thread per lipid of the pairs");
+__global__ void __launch_bounds__(MDAS_THREADS) k_mdas_select(const SysDev *__restrict__ sys, int n_pairs, int max_tries,
+                                                              int mode, const int *__restrict__ leaf) {
+    constexpr unsigned FULL = 0xffffffffu;
     const SysDev &S = sys[blockIdx.x];
     const Params &P = *S.p;
     Counters &C = *S.c;
-    if (threadIdx.x != 0) return;
-    int np = 0;
+    __shared__ int pairs[2 * MAX_PAIRS];
+    __shared__ int n_sel;
+    const int t = threadIdx.x, lane = t & 31;
     if (mode == 1) {
-        np = C.n_pairs;
-    } else {
+        if (t < 2 * C.n_pairs) pairs[t] = C.pairs[t];
+        if (t == 0) n_sel = C.n_pairs;
+    } else if (t < 32) {
         const uint32_t tag = mode == 2 ? TAG_LEAFLET : TAG_MDAS_PAIR;
-        for (int j = 0; j < max_tries && np < n_pairs; ++j) {
-            const uint4 w = draw4(P, (uint32_t)j, (uint32_t)C.move, tag, 0u);
+        int np = 0;
+        for (int j0 = 0; j0 < max_tries && np < n_pairs; j0 += 32) {
+            const uint4 w = draw4(P, (uint32_t)(j0 + lane), (uint32_t)C.move, tag, 0u);
             const int a = pick(w.x, P.n_lip), b = pick(w.y, P.n_lip);
-            if (a == b || S.ltype[a] == S.ltype[b]) continue;
-            if (mode == 2 && !(leaf[a] == 0 && leaf[b] == 1)) continue;
-            bool used = false;
-            for (int k = 0; k < 2 * np && !used; ++k) used = C.pairs[k] == a || C.pairs[k] == b;
-            if (used) continue;
-            C.pairs[2 * np] = a;
-            C.pairs[2 * np + 1] = b;
-            ++np;
-        }
-        C.n_pairs = np;
-    }
-    for (int p = 0; p < np; ++p)
-        for (int side = 0; side < 2; ++side) {
-            const int l = C.pairs[2 * p + side], o = C.pairs[2 * p + 1 - side];
-            const int tnew = S.ltype[o];
-            for (int k = 0; k < P.bpl; ++k) {
-                const int id = l * P.bpl + k;
-                const uint32_t m = S.pos[id].w;
-                set_meta(S, P, id, meta_make(meta_ta(m), P.lbt[tnew * 16 + k], k, l + 1));
+            bool ok = j0 + lane < max_tries && a != b && S.ltype[a] != S.ltype[b];
+            if (mode == 2) ok = ok && leaf[a] == 0 && leaf[b] == 1;
+            for (unsigned left = __ballot_sync(FULL, ok); left && np < n_pairs; left &= left - 1u) {
+                const int src = __ffs(left) - 1;
+                const int ca = __shfl_sync(FULL, a, src), cb = __shfl_sync(FULL, b, src);
+                bool used = false;
+                for (int k = lane; k < 2 * np; k += 32) used = used || pairs[k] == ca || pairs[k] == cb;
+                if (__any_sync(FULL, used)) continue;
+                if (lane == 0) { pairs[2 * np] = ca; pairs[2 * np + 1] = cb; }
+                __syncwarp();
+                ++np;
             }
         }
-    C.w = 0.0;
+        for (int k = lane; k < 2 * np; k += 32) C.pairs[k] = pairs[k];
+        if (lane == 0) C.n_pairs = n_sel = np;
+    }
+    __syncthreads();
+    for (int x = t; x < 2 * n_sel * P.bpl; x += MDAS_THREADS) {
+        const int y = x / P.bpl, k = x - y * P.bpl;          // lipid pairs[y] takes the type of its partner
+        const int l = pairs[y], id = l * P.bpl + k;
+        set_meta(S, P, id, meta_make(meta_ta(S.pos[id].w), P.lbt[S.ltype[pairs[y ^ 1]] * 16 + k], k, l + 1));
+    }
+    if (t == 0) C.w = 0.0;
 }
 
 void launch_mdas_select(const LaunchCtx &L, int n_pairs, int max_tries, int mode, const int *leaf) {
-    k_mdas_select<<<L.n_sys, 32, 0, L.stream>>>(L.sys, n_pairs, max_tries, mode, leaf);
+    k_mdas_select<<<L.n_sys, MDAS_THREADS, 0, L.stream>>>(L.sys, n_pairs, max_tries, mode, leaf);
 }
 
 // Leaflet of every lipid of system 0: 0 when its head (local index head_k)
@@ -448,39 +457,40 @@ void launch_mdas_dE(const LaunchCtx &L, double dlambda) {
 
 // Eq. 3: accept with min(1, exp(-w/kT)), i.e. w + kT ln u <= 0, u from
 // Philox (0, move, TAG_MDAS_ACC, 0) words 2-3.
-__global__ void k_mdas_accept(const SysDev *__restrict__ sys) {
+__global__ void __launch_bounds__(MDAS_THREADS) k_mdas_accept(const SysDev *__restrict__ sys) {
     const SysDev &S = sys[blockIdx.x];
     const Params &P = *S.p;
     Counters &C = *S.c;
-    if (threadIdx.x != 0) return;
-    const uint4 w = draw4(P, 0u, (uint32_t)C.move, TAG_MDAS_ACC, 0u);
-    const double u = unit53(w.z, w.w);
-    const int acc = (C.n_pairs > 0) && (C.w + P.kT * log(u) <= 0.0);
-    S.result[9] = u;
-    C.mdas_accept = acc;
-    if (acc) {
-        int newt[2 * MAX_PAIRS];
-        for (int p = 0; p < C.n_pairs; ++p) {
-            newt[2 * p] = S.ltype[C.pairs[2 * p + 1]];
-            newt[2 * p + 1] = S.ltype[C.pairs[2 * p]];
-        }
-        for (int x = 0; x < 2 * C.n_pairs; ++x) {
-            const int l = C.pairs[x];
-            S.ltype[l] = newt[x];
-            for (int k = 0; k < P.bpl; ++k) {
-                const int bt = P.lbt[newt[x] * 16 + k];
-                set_meta(S, P, l * P.bpl + k, meta_make(bt, bt, k, l + 1));
-            }
+    __shared__ int newt[2 * MAX_PAIRS];
+    __shared__ int accept;
+    const int t = threadIdx.x, n = 2 * C.n_pairs;
+    if (t == 0) {
+        const uint4 w = draw4(P, 0u, (uint32_t)C.move, TAG_MDAS_ACC, 0u);
+        const double u = unit53(w.z, w.w);
+        accept = C.n_pairs > 0 && C.w + P.kT * log(u) <= 0.0;
+        S.result[9] = u;
+    }
+    if (t < n) newt[t] = S.ltype[C.pairs[t ^ 1]];
+    __syncthreads();
+    if (accept) {
+        if (t < n) S.ltype[C.pairs[t]] = newt[t];
+        for (int x = t; x < n * P.bpl; x += MDAS_THREADS) {
+            const int y = x / P.bpl, k = x - y * P.bpl, l = C.pairs[y];
+            const int bt = P.lbt[newt[y] * 16 + k];
+            set_meta(S, P, l * P.bpl + k, meta_make(bt, bt, k, l + 1));
         }
     }
-    C.move++;
-    C.moves++;
-    C.moves_accepted += acc;
-    C.in_at = 0;
-    C.lambda = 0.0;
+    if (t == 0) {
+        C.mdas_accept = accept;
+        C.move++;
+        C.moves++;
+        C.moves_accepted += accept;
+        C.in_at = 0;
+        C.lambda = 0.0;
+    }
 }
 
-void launch_mdas_accept(const LaunchCtx &L) { k_mdas_accept<<<L.n_sys, 32, 0, L.stream>>>(L.sys); }
+void launch_mdas_accept(const LaunchCtx &L) { k_mdas_accept<<<L.n_sys, MDAS_THREADS, 0, L.stream>>>(L.sys); }
 
 template <typename V4>
 __global__ void k_restore(const SysDev *__restrict__ sys, const int2 *__restrict__ bmap) {
@@ -521,30 +531,26 @@ void launch_snapshot(const LaunchCtx &L) {
 // Hypothetical collective type change: lipids C.pairs[0..n) get the types in
 // C.pairs[MAX_PAIRS..MAX_PAIRS+n) as B types; dE = U_B - U_A into result[8];
 // the B marks are removed again afterwards.
-__global__ void k_mark_b(const SysDev *__restrict__ sys, int n, int clear) {
+__global__ void __launch_bounds__(MDAS_THREADS) k_mark_b(const SysDev *__restrict__ sys, int n, int clear) {
     const SysDev &S = sys[blockIdx.x];
     const Params &P = *S.p;
     Counters &C = *S.c;
-    if (threadIdx.x != 0) return;
-    for (int x = 0; x < n; ++x) {
-        const int l = C.pairs[x];
-        for (int k = 0; k < P.bpl; ++k) {
-            const int id = l * P.bpl + k;
-            const uint32_t m = S.pos[id].w;
-            const int tb = clear ? meta_ta(m) : (int)P.lbt[C.pairs[MAX_PAIRS + x] * 16 + k];
-            const uint32_t nm = meta_make(meta_ta(m), tb, k, l + 1);
-            set_meta(S, P, id, nm);
-            S.spos[S.sidx[id]].w = nm;
-        }
+    for (int x = threadIdx.x; x < n * P.bpl; x += MDAS_THREADS) {
+        const int y = x / P.bpl, k = x - y * P.bpl, l = C.pairs[y], id = l * P.bpl + k;
+        const uint32_t m = S.pos[id].w;
+        const int tb = clear ? meta_ta(m) : (int)P.lbt[C.pairs[MAX_PAIRS + y] * 16 + k];
+        const uint32_t nm = meta_make(meta_ta(m), tb, k, l + 1);
+        set_meta(S, P, id, nm);
+        S.spos[S.sidx[id]].w = nm;
     }
 }
 
 void launch_delta_energy(const LaunchCtx &L, int n) {
-    k_mark_b<<<L.n_sys, 32, 0, L.stream>>>(L.sys, n, 0);
+    k_mark_b<<<L.n_sys, MDAS_THREADS, 0, L.stream>>>(L.sys, n, 0);
     dim3 g(2 * MAX_PAIRS, L.n_sys);
     k_mdas_dE<<<g, 128, 0, L.stream>>>(L.sys, n);
     k_mdas_accumulate<<<L.n_sys, 32, 0, L.stream>>>(L.sys, 0.0, n, 0);
-    k_mark_b<<<L.n_sys, 32, 0, L.stream>>>(L.sys, n, 1);
+    k_mark_b<<<L.n_sys, MDAS_THREADS, 0, L.stream>>>(L.sys, n, 1);
 }
 
 // ------------------------------------------- trials in order, many per launch
