@@ -1323,6 +1323,8 @@ __device__ void run_partitioned(const RunArgs &a, int gid, const Grp &g, StepSme
     if (g.t == 0) base = *(volatile const unsigned *)&sb->base;
     auto bar = [&]() { return sys_barrier(sb, base, passes, ng, a.rs, g, ok); };
     auto build = [&](int par) { return part_build<G>(a, R, S, par, lg, g, bsm, sb, base, passes, ok); };
+    // closes before this launch (its first starts after the first step's barrier)
+    const unsigned long long close0 = *(volatile const unsigned long long *)&C.close_seq;
     bool tab = true;                           // the pair tables must be (re)loaded into shared memory
     if (*(volatile const int *)&C.nl_stale) {  // lists made stale outside the kernel
         if (!build(C.nl_par & 1)) return;
@@ -1330,14 +1332,23 @@ __device__ void run_partitioned(const RunArgs &a, int gid, const Grp &g, StepSme
         if (lg == 0 && g.t == 0) C.nl_builds++;
     }
     constexpr bool PC = LAM == 3;
+    // the close on the system's last group: where no trial follows a step, beside
+    // the next step's items (see k_md_run), which spares a barrier (5 systems of
+    // 128 to 700 lipids, 15 steps and 10 trials: 920 to 864 us)
+    auto close = [&](int s) {
+        if (lg == ng - 1 && g.t < 32) nl_step_close<Real, PC>(S, g.t, (C.nl_par + s) & 1);
+    };
+    bool closed = true;
     for (int s = 0; s < a.n_steps; ++s) {
+        const PipeWait pw{close0 + (unsigned long long)s, 0ull, 0u, !closed, 0};
+        if (!closed) close(s - 1);
         for (int it = lg; it < R.nln; it += ng) {
             if (tab) {
                 load_system<Real, G, false>(S, g, ssm);
                 g.sync();
                 tab = false;
             }
-            nl_step_item<Real, LAM, G, false>(a.nlmap[R.nl0 + it].y, (C.nl_par + s) & 1, &C.nl_violp[s % 3], g, ssm);
+            nl_step_item<Real, LAM, G, false>(a.nlmap[R.nl0 + it].y, (C.nl_par + s) & 1, &C.nl_violp[s % 3], g, ssm, &pw);
         }
         // the flag of step s + 1 (last read at step s - 2, before the previous barrier)
         if (lg == 0 && g.t == 0) {
@@ -1350,7 +1361,8 @@ __device__ void run_partitioned(const RunArgs &a, int gid, const Grp &g, StepSme
             tab = true;
             if (lg == 0 && g.t == 0) C.nl_builds++;
         }
-        if ((LAM == 1 || LAM == 2) && a.lam_M > 0 && (a.lam_off + s + 1) % a.lam_M == 0) {
+        const bool lam_end = (LAM == 1 || LAM == 2) && a.lam_M > 0 && (a.lam_off + s + 1) % a.lam_M == 0;
+        if (lam_end) {
             // the end of a lambda block (Eq. 2): each lipid's work term at the
             // block's last coordinates, then w += dlam * their ordered sum
             const int blk = (a.lam_off + s + 1) / a.lam_M;
@@ -1368,8 +1380,12 @@ __device__ void run_partitioned(const RunArgs &a, int gid, const Grp &g, StepSme
                 C.lambda = (double)blk * a.dlam;
             }
         }
-        // the close on the system's last group, the trial parts from its first
-        if (lg == ng - 1 && g.t < 32) nl_step_close<Real, PC>(S, g.t, (C.nl_par + s) & 1);
+        closed = s + 1 == a.n_steps || (a.swap_every > 0 && (s + 1 + a.trial_off) % a.swap_every == 0);
+        if (!closed) {
+            if (lam_end && !bar()) return;
+            continue;
+        }
+        close(s);                              // (the trial parts start from the first group)
         if (a.swap_every > 0 && (s + 1 + a.trial_off) % a.swap_every == 0) {
             for (int p = lg; p < TRIAL_PARTS; p += ng) {
                 trial_nl_part<G>(S, p, (C.nl_par + s + 1) & 1, g, tsm, false);
@@ -1417,11 +1433,21 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_md_part(const __grid_constan
 // again with the new types.  The arithmetic is that of the sequential order
 // (close and trial after the step's barrier, then a second barrier), which
 // runs otherwise.  Per step: items, barrier, list builds called for by the
-// step's displacements.  The mode is a template parameter (PIPE; the host
-// decides it by md_run_pipe): each kernel asks for its own shared memory, and
-// the other mode's code takes no registers.
-template <typename Real, int LAM, int G, bool PIPE>
+// step's displacements.
+//
+// A lone system with more items than that goes through them in turns, and
+// closes beside the next step's items too where no trial follows a step (the
+// last group does it first; it has an item less than others unless they divide
+// evenly): one barrier for such a step instead of two (10 steps at 4608 lipids: 843 to 816
+// us; a trial every third step at 2000: 885 to 841).
+//
+// The mode is a template parameter (RunMode; the host decides it by
+// md_run_mode): each kernel asks for its own shared memory, and the other
+// modes' code takes no registers.
+enum RunMode { RUN_BATCH, RUN_LONE, RUN_OVERLAPPED };
+template <typename Real, int LAM, int G, int MODE>
 __global__ void __launch_bounds__(RUN_THREADS, 1) k_md_run(const __grid_constant__ RunArgs a) {
+    constexpr bool PIPE = MODE == RUN_OVERLAPPED;
     extern __shared__ __align__(16) unsigned char dsm[];
     const int group = threadIdx.x / GRP;
     const Grp g{(int)threadIdx.x % GRP, 1 + group};
@@ -1432,15 +1458,16 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_md_run(const __grid_constant
     BuildSmem &bsm = *reinterpret_cast<BuildSmem *>(gsm);
     TrialSmem &tsm = *reinterpret_cast<TrialSmem *>(gsm);
 
-    constexpr bool pipe = PIPE;
+    constexpr bool pipe = PIPE, lone = MODE == RUN_LONE;
     const int dg = ngr - 1 - gid;                // the last gids: trial parts, then closes
     const int ptrial = pipe && dg < TRIAL_PARTS * a.n_sys ? dg : -1;
-    const int pclose = pipe && ptrial < 0 && dg < (TRIAL_PARTS + 1) * a.n_sys ? dg - TRIAL_PARTS * a.n_sys : -1;
+    const int pclose = lone ? (dg == 0 ? 0 : -1)
+                       : pipe && ptrial < 0 && dg < (TRIAL_PARTS + 1) * a.n_sys ? dg - TRIAL_PARTS * a.n_sys : -1;
     // an item's system before any close, trial or mark of this launch (those
     // start after the first barrier)
     unsigned long long close0 = 0, trial0 = 0;
     unsigned mark0 = 0;
-    if (pipe && gid < a.n_nl) {
+    if ((pipe || lone) && gid < a.n_nl) {
         const Counters &C = *a.sys[a.nlmap[gid].x].c;
         close0 = *(volatile const unsigned long long *)&C.close_seq;
         trial0 = *(volatile const unsigned long long *)&C.trial;
@@ -1462,6 +1489,7 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_md_run(const __grid_constant
     for (int s = 0; s < a.n_steps; ++s) {
         // a trial after step s - 1: the ordinal o of that trial in this launch
         const bool tprev = s > 0 && a.swap_every > 0 && (s + a.trial_off) % a.swap_every == 0;
+        const bool tnext = a.swap_every > 0 && (s + 1 + a.trial_off) % a.swap_every == 0;
         if (pipe) {
             if (gid < a.n_nl) {
                 const int2 bm = a.nlmap[gid];
@@ -1489,6 +1517,14 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_md_run(const __grid_constant
                 nl_step_close<Real, LAM == 3>(S, g.t, (S.c->nl_par + s - 1) & 1);
             }
         } else {
+            PipeWait pw;
+            pw.has_close = lone && s > 0 && !tprev;
+            pw.close_target = close0 + (unsigned long long)s;
+            pw.has_trial = 0;
+            if (lone && pclose >= 0 && pw.has_close && g.t < 32) {
+                const SysDev &S = a.sys[pclose];
+                nl_step_close<Real, LAM == 3>(S, g.t, (S.c->nl_par + s - 1) & 1);
+            }
             for (int it = gid; it < a.n_nl; it += ngr) {
                 const int2 bm = a.nlmap[it];
                 const SysDev &S = a.sys[bm.x];
@@ -1497,7 +1533,8 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_md_run(const __grid_constant
                     g.sync();
                     tab_sys = bm.x;
                 }
-                nl_step_item<Real, LAM, G, PIPE>(bm.y, (S.c->nl_par + s) & 1, &S.c->nl_violp[s % 3], g, ssm);
+                nl_step_item<Real, LAM, G, PIPE>(bm.y, (S.c->nl_par + s) & 1, &S.c->nl_violp[s % 3], g, ssm,
+                                                 lone ? &pw : nullptr);
             }
         }
         // the flag of step s + 1 (last read at step s - 2, before the previous barrier)
@@ -1540,9 +1577,9 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_md_run(const __grid_constant
                     C.w += a.sys[q].p->sc_delta > 0.0 ? sum : a.dlam * sum;
                     C.lambda = (double)blk * a.dlam;
                 }
-            if (pipe && !grid_barrier(a.rs, bs)) return;
+            if ((pipe || (lone && !tnext)) && !grid_barrier(a.rs, bs)) return;
         }
-        if (!pipe) {
+        if (!pipe && (!lone || tnext)) {
             // the close of system q on block gridDim - 1 - q % gridDim (the
             // trial parts start on the first blocks, so both overlap)
             if (threadIdx.x < 32)
@@ -1550,7 +1587,7 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_md_run(const __grid_constant
                     const SysDev &S = a.sys[q];
                     nl_step_close<Real, LAM == 3>(S, threadIdx.x, (S.c->nl_par + s) & 1);
                 }
-            if (a.swap_every > 0 && (s + 1 + a.trial_off) % a.swap_every == 0) {
+            if (tnext) {
                 for (int it = gid; it < TRIAL_PARTS * a.n_sys; it += ngr) {
                     const SysDev &S = a.sys[it / TRIAL_PARTS];
                     trial_nl_part<G>(S, it % TRIAL_PARTS, (S.c->nl_par + s + 1) & 1, g, tsm, false);
@@ -1560,14 +1597,14 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_md_run(const __grid_constant
             if (!grid_barrier(a.rs, bs)) return;
         }
     }
-    if (pipe && a.n_steps > 0) {
-        // the last step's close and trial, then a barrier
+    // the last step's close and trial, then a barrier
+    if (a.n_steps > 0 && (pipe || (lone && !(a.swap_every > 0 && (a.n_steps + a.trial_off) % a.swap_every == 0)))) {
         const int s = a.n_steps;
         if (pclose >= 0 && g.t < 32) {
             const SysDev &S = a.sys[pclose];
             nl_step_close<Real, LAM == 3>(S, g.t, (S.c->nl_par + s - 1) & 1);
         }
-        if (ptrial >= 0 && a.swap_every > 0 && (s + a.trial_off) % a.swap_every == 0) {
+        if (pipe && ptrial >= 0 && a.swap_every > 0 && (s + a.trial_off) % a.swap_every == 0) {
             const SysDev &S = a.sys[ptrial / TRIAL_PARTS];
             trial_nl_part<G>(S, ptrial % TRIAL_PARTS, (S.c->nl_par + s) & 1, g, tsm, false);
         }
@@ -1584,10 +1621,11 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_md_run(const __grid_constant
         }
 }
 
-// Whether a launch of n_blocks persistent blocks over n_items step items of
-// n_sys systems runs in overlapped mode (see k_md_run).
-inline bool md_run_pipe(int n_items, int n_sys, int n_blocks) {
-    return n_items + (TRIAL_PARTS + 1) * n_sys <= n_blocks * RUN_GROUPS;
+// How a launch of n_blocks persistent blocks over n_items step items of n_sys
+// systems runs (see k_md_run).
+inline RunMode md_run_mode(int n_items, int n_sys, int n_blocks) {
+    if (n_items + (TRIAL_PARTS + 1) * n_sys <= n_blocks * RUN_GROUPS) return RUN_OVERLAPPED;
+    return n_sys == 1 ? RUN_LONE : RUN_BATCH;
 }
 
 template <typename Real, int LAM, int G>
@@ -1609,22 +1647,26 @@ static cudaError_t run_launch(const LaunchCtx &L, int n_steps, int swap_every, i
     a.n_steps = n_steps; a.swap_every = swap_every; a.trial_off = trial_off; a.rs = rs;
     a.lam_M = lam_M; a.lam_off = lam_off; a.dlam = dlam;
     void *args[] = {&a};
-    const bool pipe = !a.gsys && md_run_pipe(a.n_nl, a.n_sys, n_blocks);
-    const void *fn = a.gsys ? (const void *)k_md_part<Real, LAM, G>
-                     : pipe ? (const void *)k_md_run<Real, LAM, G, true> : (const void *)k_md_run<Real, LAM, G, false>;
+    const RunMode mode = a.gsys ? RUN_BATCH : md_run_mode(a.n_nl, a.n_sys, n_blocks);
+    const bool pipe = mode == RUN_OVERLAPPED;
+    const void *fn = a.gsys                ? (const void *)k_md_part<Real, LAM, G>
+                     : pipe                ? (const void *)k_md_run<Real, LAM, G, RUN_OVERLAPPED>
+                     : mode == RUN_LONE    ? (const void *)k_md_run<Real, LAM, G, RUN_LONE>
+                                           : (const void *)k_md_run<Real, LAM, G, RUN_BATCH>;
     return cudaLaunchCooperativeKernel(fn, dim3(n_blocks), dim3(RUN_THREADS), args,
                                        RUN_GROUPS * (pipe ? group_smem<Real, G, true>() : group_smem<Real, G, false>()),
                                        L.stream);
 }
 
-// Shared-memory limits of the three kernels, and whether a block of each fits
+// Shared-memory limits of the kernels, and whether a block of each fits
 // on an SM.  No more shared memory than a block needs: the rest of the SM's
 // 256 KB stays L1 cache for the step's position gathers.
 template <typename Real, int LAM, int G>
 static cudaError_t run_setup(int *blocks_per_sm) {
     const struct { const void *fn; size_t smem; } kernels[] = {
-        {(const void *)k_md_run<Real, LAM, G, true>, RUN_GROUPS * group_smem<Real, G, true>()},
-        {(const void *)k_md_run<Real, LAM, G, false>, RUN_GROUPS * group_smem<Real, G, false>()},
+        {(const void *)k_md_run<Real, LAM, G, RUN_OVERLAPPED>, RUN_GROUPS * group_smem<Real, G, true>()},
+        {(const void *)k_md_run<Real, LAM, G, RUN_LONE>, RUN_GROUPS * group_smem<Real, G, false>()},
+        {(const void *)k_md_run<Real, LAM, G, RUN_BATCH>, RUN_GROUPS * group_smem<Real, G, false>()},
         {(const void *)k_md_part<Real, LAM, G>, RUN_GROUPS * group_smem<Real, G, false>()}};
     int dev = 0, maxsm = 0;
     cudaGetDevice(&dev);
