@@ -17,6 +17,7 @@
 #include <cstdio>
 
 #include "mdas_phys.cuh"
+#include "mdas_trial.cuh"
 
 namespace mdas {
 
@@ -417,7 +418,7 @@ __global__ void __launch_bounds__(PAIR_THREADS, 8) k_pair(const SysDev *__restri
                 r2inv = (Real)r2i;
                 rinv = (Real)rsqrtf((float)r2);
             } else {
-                rinv = (Real)(1.0 / sqrt((double)r2));
+                rinv = (Real)rsqrt_near((double)r2, (float)r2);
                 r2inv = rinv * rinv;
                 r6inv = r2inv * r2inv * r2inv;
             }
@@ -628,8 +629,7 @@ __global__ void __launch_bounds__(BEAD_BLOCK) k_bonded_energy(const SysDev *__re
 // wait in a ring until 32 are there, and then each lane takes one through FP64.
 //
 // The FP64 pipe bounds it (two operations per clock and SM): each pair goes
-// through it once, at about 27 operations with 1/r from a float seed and two
-// Newton steps, the last in the residual form (within an ulp), where the force
+// through it once, at about 20 operations with 1/r from rsqrt_near, where the force
 // kernel's pass took every pair twice with a square root, a division and the
 // forces (a call for forces and energies, 1152 lipids: 654 to 334 us).
 constexpr int ENERGY_WARPS = 4;
@@ -670,21 +670,22 @@ __global__ void __launch_bounds__(32 * ENERGY_WARPS) k_cell_energy(const SysDev 
     const int first_of = first - off;             // place of candidate t of cell q: t + first_of
     const int i0 = __shfl_sync(FULL, first, 0), ni = __shfl_sync(FULL, cnt, 0);
     const float q0 = P.qsf[0], q1 = P.qsf[1], q2 = P.qsf[2], rc2f = P.rc2f;
-    double elj = 0.0, erf = 0.0, pairs = 0.0;
+    double elj = 0.0, erf = 0.0;
+    int pairs = 0;
     int head = 0, tail = 0;
     auto evaluate = [&](int nt) {
         if (lane < nt) {
             const int4 e = ring[w][(head + lane) & 63];
             const double x = (double)e.x * P.qs[0], y = (double)e.y * P.qs[1], z = (double)e.z * P.qs[2];
             const double r2 = fma(x, x, fma(y, y, z * z));
-            if (r2 < P.rc2) {
-                double ri = (double)rsqrtf((float)r2);
-                ri = ri * fma(-0.5 * r2, ri * ri, 1.5);
-                ri = fma(0.5 * ri, fma(-(r2 * ri), ri, 1.0), ri);
+            const float fx = (float)e.x * q0, fy = (float)e.y * q1, fz = (float)e.z * q2;
+            const float r2f = fx * fx + fy * fy + fz * fz;
+            if (inside_rc(P, r2, r2f)) {
+                const double ri = rsqrt_near(r2, r2f);
                 const double r2i = ri * ri, r6 = r2i * r2i * r2i;
                 elj += fma(fma(P.c12[e.w], r6, -P.c6[e.w]), r6, -P.ush[e.w]);
                 erf = fma(P.qq[e.w], fma(P.krf, r2, ri - P.crf), erf);
-                pairs += 1.0;
+                ++pairs;
             }
         }
         head += nt;
@@ -735,7 +736,7 @@ __global__ void __launch_bounds__(32 * ENERGY_WARPS) k_cell_energy(const SysDev 
     if (lane == 0) {
         S.epart[4 * c + 0] = elj;
         S.epart[4 * c + 1] = erf;
-        S.epart[4 * c + 2] = pairs;
+        S.epart[4 * c + 2] = (double)pairs;
     }
 }
 

@@ -6,18 +6,39 @@
 
 namespace mdas {
 
+// 1/sqrt(r2) in FP64 from a float r2f near r2 (relative difference below
+// 2^-21): the float function's value, widened by its bits, and one third-order
+// step, y (1 + e/2 + 3 e^2/8) with e = 1 - r2 y^2 below 2^-19 (what it leaves out
+// is below 2^-58): within an ulp of FP64, as the square root and the division.
+// The FP64 pipe takes two operations per clock and SM and bounds every sum over
+// pairs in FP64; this takes five of them, two Newton steps and the conversions
+// to and from float took ten: 20 FP64 steps at 128 lipids 996 to 895 us, 256
+// exchange trials at 1424 lipids 537 to 501, 20 FP32 steps with a trial each at
+// 1152 lipids 571 to 561.
+__device__ __forceinline__ double rsqrt_near(double r2, float r2f) {
+    const unsigned b = __float_as_uint(rsqrtf(r2f));          // positive and normal
+    const double y = __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
+    const double e = fma(-(r2 * y), y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
+// Whether a pair at r2 (and r2f in FP32) that passed the FP32 test of the
+// cutoff is inside it: FP64 decides within float rounding of it only.
+template <class Pm>
+__device__ __forceinline__ bool inside_rc(const Pm &P, double r2, float r2f) {
+    return r2f < P.rc2f_lo || r2 < P.rc2;
+}
+
 // FP64 change of one pair's energy (LJ with potential shift + reaction field)
-// when its type pair goes from (oi, oj) to (ni, nj), at squared distance r2;
-// 1/r from a float seed refined by two Newton steps (no FP64 divide or sqrt).
-__device__ __forceinline__ double pair_du(const Params &P, int oi, int oj, int ni, int nj, double r2) {
+// when its type pair goes from (oi, oj) to (ni, nj), at squared distance r2
+// (r2f in FP32).
+__device__ __forceinline__ double pair_du(const Params &P, int oi, int oj, int ni, int nj, double r2, float r2f) {
     const int xo = oi * 16 + oj, xn = ni * 16 + nj;
-    double ri = (double)rsqrtf((float)r2);
-    ri = ri * (1.5 - 0.5 * r2 * ri * ri);
-    ri = ri * (1.5 - 0.5 * r2 * ri * ri);
+    const double ri = rsqrt_near(r2, r2f);
     const double r2i = ri * ri;
     const double r6 = r2i * r2i * r2i;
-    return (P.c12[xn] - P.c12[xo]) * r6 * r6 - (P.c6[xn] - P.c6[xo]) * r6 - (P.ush[xn] - P.ush[xo]) +
-           (P.qq[xn] - P.qq[xo]) * (ri + P.krf * r2 - P.crf);
+    const double lj = fma(fma(P.c12[xn] - P.c12[xo], r6, -(P.c6[xn] - P.c6[xo])), r6, -(P.ush[xn] - P.ush[xo]));
+    return fma(P.qq[xn] - P.qq[xo], fma(P.krf, r2, ri - P.crf), lj);
 }
 
 // Metropolis test of Eq. 1, accept iff dE + kT ln u <= 0, decided as in FP64:
@@ -148,11 +169,11 @@ __device__ __forceinline__ double trial_entry(const SysDev &S, int a, int b, con
     const bool chj = (lj == a || lj == b) && ((sm.m >> kjl) & 1);
     if (chj && lj * P.bpl + kjl < sm.chg_id[ci]) return 0.0;   // a changed pair once, by the lower id
     const double ex = (double)ix * P.qs[0], ey = (double)iy * P.qs[1], ez = (double)iz * P.qs[2];
-    const double r2 = ex * ex + ey * ey + ez * ez;
-    if (r2 >= P.rc2) return 0.0;
+    const double r2 = fma(ex, ex, fma(ey, ey, ez * ez));
+    if (!inside_rc(P, r2, r2f)) return 0.0;
     const int old_j = meta_ta(pj.w);
     const int new_j = chj ? (int)P.lbt[(lj == a ? sm.tb : sm.ta) * 16 + kjl] : old_j;
-    return pair_du(P, sm.chg_old[ci], old_j, sm.chg_new[ci], new_j, r2);
+    return pair_du(P, sm.chg_old[ci], old_j, sm.chg_new[ci], new_j, r2, r2f);
 }
 
 // Part p (of TRIAL_PARTS) of one exchange trial from the pair list (valid
@@ -252,11 +273,9 @@ __device__ __forceinline__ double lj_soft(const Params &P, int x, double r2, dou
 // U_l1 - U_l0 with the Lennard-Jones parts from Eq. 4 for both end states and
 // the reaction field linear in lambda.
 __device__ __forceinline__ double pair_dw_soft(const Params &P, int oi, int oj, int ni, int nj, double r2,
-                                               double l0, double l1) {
+                                               float r2f, double l0, double l1) {
     const int xo = oi * 16 + oj, xn = ni * 16 + nj;
-    double ri = (double)rsqrtf((float)r2);
-    ri = ri * (1.5 - 0.5 * r2 * ri * ri);
-    ri = ri * (1.5 - 0.5 * r2 * ri * ri);
+    const double ri = rsqrt_near(r2, r2f);
     const double lj = (lj_soft(P, xo, r2, 1.0 - l1) + lj_soft(P, xn, r2, l1)) -
                       (lj_soft(P, xo, r2, 1.0 - l0) + lj_soft(P, xn, r2, l0));
     return lj + (l1 - l0) * (P.qq[xn] - P.qq[xo]) * (ri + P.krf * r2 - P.crf);
@@ -299,9 +318,10 @@ __device__ inline double mdas_work_part(const SysDev &S, int x, int par, const G
                 const int oj = meta_ta(pj.w), nj = meta_tb(pj.w);
                 if (oj != nj && meta_lip(pj.w) * P.bpl + meta_k(pj.w) < i) continue;
                 const double ex = (double)ix * P.qs[0], ey = (double)iy * P.qs[1], ez = (double)iz * P.qs[2];
-                const double r2 = ex * ex + ey * ey + ez * ez;
-                if (r2 >= P.rc2) continue;
-                acc += P.sc_delta > 0.0 ? pair_dw_soft(P, oi, oj, ni, nj, r2, l0, l1) : pair_du(P, oi, oj, ni, nj, r2);
+                const double r2 = fma(ex, ex, fma(ey, ey, ez * ez));
+                if (!inside_rc(P, r2, r2f)) continue;
+                acc += P.sc_delta > 0.0 ? pair_dw_soft(P, oi, oj, ni, nj, r2, r2f, l0, l1)
+                                        : pair_du(P, oi, oj, ni, nj, r2, r2f);
             }
         }
     }

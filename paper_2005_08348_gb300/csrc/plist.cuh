@@ -644,8 +644,7 @@ __device__ __forceinline__ void nl_step_item(int k0, int par, int *viol, const G
         asm volatile("cp.async.commit_group;\n" ::: "memory");
     }
 
-    const Real rc2 = F32 ? (Real)P.rc2f : (Real)P.rc2;
-    const Real rc2lo = F32 ? (Real)P.rc2f_lo : (Real)P.rc2;
+    const Real rc2 = (Real)P.rc2f, rc2lo = (Real)P.rc2f_lo;
     const Real krf2 = F32 ? (Real)P.krf2f : (Real)(2.0 * P.krf);
     // LAM: 0 no alchemical path, 1 linear path, 2 soft-core path (Eq. 4),
     // 3 no alchemical path, with the pressure coupling's virial sums and -M v term
@@ -665,7 +664,7 @@ __device__ __forceinline__ void nl_step_item(int k0, int par, int *viol, const G
     // FP32, whether r^2 lies within float rounding of it (decided from the
     // exact offsets by in_exact; about one entry in 2 * 10^4).  A partner at
     // zero distance (a padding entry is the bead itself) is outside.
-    struct Sep { Real x, y, z, r2; uint32_t w; bool in, edge; };
+    struct Sep { Real x, y, z, r2; float r2f; uint32_t w; bool in, edge; };
     auto cull = [&](uint4 pj) {
         Sep e;
         const int ix = (int)(pi.x - pj.x), iy = (int)(pi.y - pj.y), iz = (int)(pi.z - pj.z);
@@ -680,8 +679,14 @@ __device__ __forceinline__ void nl_step_item(int k0, int par, int *viol, const G
         }
         e.r2 = fmr(e.x, e.x, fmr(e.y, e.y, e.z * e.z));
         e.w = pj.w;
-        e.in = (e.r2 < rc2lo) & (e.r2 > (Real)0);
-        e.edge = F32 && (e.r2 < rc2) & !(e.r2 < rc2lo);
+        if (F32) {
+            e.in = (e.r2 < rc2lo) & (e.r2 > (Real)0);
+            e.edge = (e.r2 < rc2) & !(e.r2 < rc2lo);
+        } else {                                   // (has passed the FP32 test below)
+            const float fx = (float)ix * qs0, fy = (float)iy * qs1, fz = (float)iz * qs2;
+            e.r2f = fmaf(fx, fx, fmaf(fy, fy, fz * fz));
+            e.in = inside_rc(P, (double)e.r2, e.r2f);
+        }
         return e;
     };
     auto in_exact = [&](uint4 pj) {
@@ -716,13 +721,7 @@ __device__ __forceinline__ void nl_step_item(int k0, int par, int *viol, const G
             r2inv = (Real)r2i;
             rinv = (Real)ri;
         } else {
-            // 1/r from a float seed and two Newton steps, the second in the
-            // residual form (an error within an ulp, as the square root and the
-            // division had, at a fifth of their operations)
-            double ri = (double)rsqrtf((float)e.r2);
-            ri = ri * fma(-0.5 * (double)e.r2, ri * ri, 1.5);
-            ri = fma(0.5 * ri, fma(-((double)e.r2 * ri), ri, 1.0), ri);
-            rinv = (Real)ri;
+            rinv = (Real)rsqrt_near((double)e.r2, e.r2f);
             r2inv = rinv * rinv;
             r6inv = r2inv * r2inv * r2inv;
         }

@@ -54,11 +54,11 @@ __device__ double bead_delta(const SysDev &S, const Params &P, int i, uint4 pi, 
         if (chj && j < i) continue;
         if (li >= 0 && meta_lip(pj.w) == li && ((em >> meta_k(pj.w)) & 1u)) continue;
         const double ex = (double)ix * P.qs[0], ey = (double)iy * P.qs[1], ez = (double)iz * P.qs[2];
-        const double r2 = ex * ex + ey * ey + ez * ez;
-        if (r2 >= P.rc2) continue;
+        const double r2 = fma(ex, ex, fma(ey, ey, ez * ez));
+        if (!inside_rc(P, r2, r2f)) continue;
         const int old_j = meta_ta(pj.w);
         const int new_j = chj ? newt(pj.w, j) : old_j;
-        acc += pair_du(P, old_i, old_j, new_i, new_j, r2);
+        acc += pair_du(P, old_i, old_j, new_i, new_j, r2, r2f);
     }
     return acc;
 }
