@@ -392,9 +392,10 @@ mdas_status mdas_set_list_lanes(mdas_system *s, int32_t lanes);
  * resolves in order each one that no earlier accepted or pending trial can
  * influence (the rest are evaluated again in the next round: few rounds when
  * trials rarely meet, as in a large bilayer); MDAS_TRIALS_SEQUENTIAL runs
- * them one after another from the pair lists, every system of a batch at
- * once (one launch per trial, no rounds: better where trials keep meeting, as
- * in small bilayers); MDAS_TRIALS_AUTO (the default) runs them sequentially
+ * them in order from the pair lists, every system of a batch at once (up to
+ * 256 trials per launch, evaluated beside each other and walked in order, no
+ * rounds: better where trials keep meeting, as in small bilayers);
+ * MDAS_TRIALS_AUTO (the default) runs them sequentially
  * unless a system of the batch has pressure coupling (its lists may predate
  * the last box update), then speculatively.  Both give the sequential
  * order's decisions (dE sums in another order, the same within rounding);

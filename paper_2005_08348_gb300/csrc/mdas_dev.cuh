@@ -27,7 +27,7 @@ constexpr int NL_BEADS_MIN = NL_BLOCK / NL_LANES_MAX;   // beads of the smallest
 __host__ __device__ constexpr bool nl_lanes_ok(int g) { return g == 2 || g == 4; }
 constexpr int NL_PART = 8;             // bonded partners per bead at most
 constexpr int NLB_BEADS = 8;           // beads of one list-build task (one warp),
-constexpr int NLB_FEW = 2;             // and where the tasks would leave most warps idle
+constexpr int NLB_FEW = 1;             // and at least, where the tasks would leave most warps idle
 constexpr int NL_BUILD_BLOCKS = 152 * 8;   // blocks of the list-build kernel (separate launches)
 // list-build tasks of a cell with the given number of beads, at most run per task
 __host__ __device__ constexpr int nl_build_tasks(int beads, int run) { return (beads + run - 1) / run; }

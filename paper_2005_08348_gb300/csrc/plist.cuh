@@ -1239,14 +1239,15 @@ static __device__ bool grid_barrier_flag(RunSync *rs, BarState &bs, const RunArg
 // List build of every system whose flag is set; buffer (nl_par + b) & 1 holds
 // the current positions.  Three barriers.
 //
-// Tasks of NLB_FEW beads while the beads still give every warp of the grid at
-// most one such task (shorter chains per warp: 25 against 33 us for the
-// 128-lipid bilayer's task phase), of NLB_BEADS beyond (fewer walks over the
-// candidates).
+// Tasks of 1, 2 or 4 beads while the beads still give every warp of the grid
+// at most about one such task (a warp's chain bounds the phase), of NLB_BEADS
+// beyond (fewer walks over the candidates).  20 steps at 700 lipids take 522 us
+// for 561 with 8, at 128 lipids 358 for 368 with 2.
 template <int NG>
 __device__ __noinline__ bool run_build(const RunArgs &a, int which, int s, int b, const Grp &g, int gid, int G, BuildSmem &sm,
                                        BarState &bs) {
-    const bool few = a.n_bead * (BEAD_BLOCK / NLB_FEW) <= (GRP / 32) * G;
+    const int beads = a.n_bead * BEAD_BLOCK, warps = (GRP / 32) * G;
+    const int run = beads <= warps ? 1 : beads <= 2 * warps ? 2 : beads <= 4 * warps ? 4 : NLB_BEADS;
     for (int it = gid; it < a.n_bead; it += G) {
         const int2 bm = a.beadmap[it];
         const SysDev &S = a.sys[bm.x];
@@ -1256,15 +1257,17 @@ __device__ __noinline__ bool run_build(const RunArgs &a, int which, int s, int b
     for (int it = gid; it < a.n_lsort; it += G) {
         const int2 bm = a.lsortmap[it];
         const SysDev &S = a.sys[bm.x];
-        if (build_flag(*S.c, which, s)) nl_place_item(S, bm.y, (S.c->nl_par + b) & 1, few ? NLB_FEW : NLB_BEADS, g, sm);
+        if (build_flag(*S.c, which, s)) nl_place_item(S, bm.y, (S.c->nl_par + b) & 1, run, g, sm);
     }
     if (!grid_barrier(a.rs, bs)) return false;
     // one warp per task, consecutive tasks on different SMs
     const int w = g.t >> 5;
     auto flag = [&](const SysDev &S) { return build_flag(*S.c, which, s) != 0; };
     auto par = [&](const SysDev &S) { return (S.c->nl_par + b) & 1; };
-    if (few) nl_build_dealt<NG, NLB_FEW>(a.sys, a.n_sys, w * G + gid, (GRP / 32) * G, g.t & 31, sm.w[w], flag, par);
-    else nl_build_dealt<NG, NLB_BEADS>(a.sys, a.n_sys, w * G + gid, (GRP / 32) * G, g.t & 31, sm.w[w], flag, par);
+    if (run == 1) nl_build_dealt<NG, 1>(a.sys, a.n_sys, w * G + gid, warps, g.t & 31, sm.w[w], flag, par);
+    else if (run == 2) nl_build_dealt<NG, 2>(a.sys, a.n_sys, w * G + gid, warps, g.t & 31, sm.w[w], flag, par);
+    else if (run == 4) nl_build_dealt<NG, 4>(a.sys, a.n_sys, w * G + gid, warps, g.t & 31, sm.w[w], flag, par);
+    else nl_build_dealt<NG, NLB_BEADS>(a.sys, a.n_sys, w * G + gid, warps, g.t & 31, sm.w[w], flag, par);
     return grid_barrier(a.rs, bs);
 }
 
