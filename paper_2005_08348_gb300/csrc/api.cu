@@ -25,7 +25,9 @@ struct Batch {
     int precision = 0;
     cudaStream_t stream = nullptr;
     int max_bead_blocks = 1;
-    int *dscratch = nullptr;      // [2]: pending sum, error or
+    int *status = nullptr;        // [2], pinned host memory that kernels write: pending sum, error or
+    Params *boxes = nullptr;      // pinned, one per system: the parameters after box updates
+    size_t boxes_cap = 0;
     unsigned int *bticket = nullptr;   // last-block ticket of the step kernel over the batch
     void *rsync = nullptr;        // grid-barrier state of the persistent MD kernel (zeroed)
     void *part = nullptr;         // partition of the persistent kernel's groups among the systems
@@ -202,7 +204,8 @@ void destroy_batch(Batch *b) {
     free_map(b->beads); free_map(b->cells); free_map(b->sortcells); free_map(b->syss);
     free_map(b->nlbeads); free_map(b->lsort);
     if (b->dsys) cudaFree(b->dsys);
-    if (b->dscratch) cudaFree(b->dscratch);
+    if (b->status) cudaFreeHost(b->status);
+    if (b->boxes) cudaFreeHost(b->boxes);
     if (b->bticket) cudaFree(b->bticket);
     if (b->rsync) cudaFree(b->rsync);
     if (b->part) cudaFree(b->part);
@@ -254,7 +257,7 @@ mdas_status make_batch(const std::vector<mdas_system *> &v, std::unique_ptr<Batc
     CK(upload_map(b->syss, mp.syss));
     CK(upload_map(b->nlbeads, mp.nlbeads));
     CK(upload_map(b->lsort, mp.lsort));
-    CK(cudaMalloc(&b->dscratch, sizeof(int) * 4));
+    CK(cudaHostAlloc((void **)&b->status, sizeof(int) * 2, cudaHostAllocMapped | cudaHostAllocPortable));
     CK(cudaMalloc(&b->bticket, sizeof(unsigned int)));
     CK(cudaMemset(b->bticket, 0, sizeof(unsigned int)));
     CK(cudaMalloc(&b->rsync, md_run_sync_bytes()));
@@ -302,7 +305,7 @@ mdas_status refill_batch(Batch &b, const std::vector<mdas_system *> &v) {
     size_t cap_syss = 0;
     if (!b.syss.d) CK(grow((void **)&b.syss.d, cap_syss, 4096, sizeof(int2)));
     if (syss.size() > 4096) return fail(s, MDAS_ERR_INVALID_ARG, "batch: more than 4096 systems");
-    if (!b.dscratch) CK(cudaMalloc(&b.dscratch, sizeof(int) * 4));
+    if (!b.status) CK(cudaHostAlloc((void **)&b.status, sizeof(int) * 2, cudaHostAllocMapped | cudaHostAllocPortable));
     if (!b.bticket) {
         CK(cudaMalloc(&b.bticket, sizeof(unsigned int)));
         CK(cudaMemset(b.bticket, 0, sizeof(unsigned int)));
@@ -348,14 +351,14 @@ __device__ void batch_status_warp(const SysDev *__restrict__ sys, int n, int *ou
 
 __global__ void k_batch_status(const SysDev *__restrict__ sys, int n, int *out) { batch_status_warp(sys, n, out); }
 
-// summed: the batch's last kernel has left the status in dscratch
+// summed: the batch's last kernel has left the status.  The kernel writes it to
+// the host's own memory, complete once the stream has drained: a copy to
+// pageable memory after it cost 6 to 10 us a call.
 mdas_status batch_status(mdas_system *s, Batch &b, int *pending, int *err, bool summed = false) {
-    if (!summed) k_batch_status<<<1, 32, 0, b.stream>>>(b.dsys, (int)b.sys.size(), b.dscratch);
-    int h[2];
-    CK(cudaMemcpyAsync(h, b.dscratch, sizeof(h), cudaMemcpyDeviceToHost, b.stream));
+    if (!summed) k_batch_status<<<1, 32, 0, b.stream>>>(b.dsys, (int)b.sys.size(), b.status);
     CK(cudaStreamSynchronize(b.stream));
-    *pending = h[0];
-    *err = h[1];
+    *pending = b.status[0];
+    *err = b.status[1];
     return MDAS_OK;
 }
 
@@ -574,7 +577,7 @@ mdas_status run_md(mdas_system *s, Batch &b, long long n_steps, int swap_every, 
             k_run_end<<<1, 32, 0, b.stream>>>(b.rsync, (int)md_run_sync_bytes(), b.dsys, (int)b.sys.size(),
                                               L.part ? (SysBar *)((char *)L.part + part_layout((int)b.sys.size(),
                                                        L.part_groups).bars) : nullptr,
-                                              summed ? b.dscratch : nullptr);
+                                              summed ? b.status : nullptr);
             launches += 1;
             if (pc_nst > 0) { launch_pcouple(L); ++launches; }
             continue;
@@ -601,23 +604,36 @@ mdas_status run_md(mdas_system *s, Batch &b, long long n_steps, int swap_every, 
         if (pc_nst > 0) { launch_pcouple(L); ++launches; }
     }
     if (pc_nst > 0) {
-        // the host copy of the box-derived parameters
-        for (auto *x : b.sys)
-            if (x->hp.pc_nst > 0) CK(cudaMemcpyAsync(&x->hp, x->hs.p, sizeof(Params), cudaMemcpyDeviceToHost, b.stream));
-        CK(cudaStreamSynchronize(b.stream));
+        // the host copy of the box-derived parameters, by way of pinned memory:
+        // one wait for it and the status
+        if (b.boxes_cap < b.sys.size()) {
+            if (b.boxes) cudaFreeHost(b.boxes);
+            b.boxes = nullptr;
+            b.boxes_cap = 0;
+            CK(cudaHostAlloc((void **)&b.boxes, sizeof(Params) * b.sys.size(), cudaHostAllocPortable));
+            b.boxes_cap = b.sys.size();
+        }
+        for (size_t k = 0; k < b.sys.size(); ++k)
+            if (b.sys[k]->hp.pc_nst > 0)
+                CK(cudaMemcpyAsync(b.boxes + k, b.sys[k]->hs.p, sizeof(Params), cudaMemcpyDeviceToHost, b.stream));
     }
     for (auto *x : b.sys) x->kernel_launches += launches;
     CK(cudaGetLastError());
     CK(tm.collect(b));
-    return check ? check_err(s, b, summed) : MDAS_OK;
+    if (pc_nst == 0) return check ? check_err(s, b, summed) : MDAS_OK;
+    const mdas_status st = check ? check_err(s, b, summed) : MDAS_OK;
+    CK(cudaStreamSynchronize(b.stream));       // (at once after check_err)
+    for (size_t k = 0; k < b.sys.size(); ++k)
+        if (b.sys[k]->hp.pc_nst > 0) b.sys[k]->hp = b.boxes[k];
+    return st;
 }
 
 // n exchange trials per system of a batch with sequential semantics.
 // The way a batch runs its exchange trials: its first system's choice, or
-// for MDAS_TRIALS_AUTO one after another from the pair lists (measured
-// faster for small and large bilayers alike: 64 replicas of 128-2048 lipids,
-// 100 trials each, 1.8 against 7.1 ms; a 4608-lipid bilayer, 1024 trials,
-// 104k against 72k trials/s) unless a system has pressure coupling, whose
+// for MDAS_TRIALS_AUTO in order from the pair lists (faster for small and
+// large bilayers alike, already with a launch per trial: 64 replicas of
+// 128-2048 lipids, 100 trials each, 1.8 against 7.1 ms; a 4608-lipid bilayer,
+// 1024 trials, 104k against 72k trials/s) unless a system has pressure coupling, whose
 // lists may predate the last box update.
 int trial_path_of(const Batch &b, int) {
     if (b.trial_path != MDAS_TRIALS_AUTO) return b.trial_path;
