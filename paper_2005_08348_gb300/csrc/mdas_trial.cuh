@@ -145,11 +145,10 @@ __device__ __forceinline__ void trial_beads(const SysDev &S, int a, int b, int t
 
 // Energy change of entry f of the trial in sm (0 outside the cutoff; a pair of
 // two changed beads counts once, by the lower id).  seen(slot): called with the
-// partner's list slot before its position is loaded; near(lipid): with the
-// lipid of a partner inside the cutoff (-1: water).
-template <int G, class Seen, class Near>
+// partner's list slot before its position is loaded.
+template <int G, class Seen>
 __device__ __forceinline__ double trial_entry(const SysDev &S, int a, int b, const uint4 *cur, const TrialSmem &sm, int f,
-                                              Seen seen, Near near) {
+                                              Seen seen) {
     const Params &P = *S.p;
     int lo = 0, hi = sm.nchg * G - 1;         // the (bead, column) holding entry f
     while (lo < hi) {
@@ -165,7 +164,6 @@ __device__ __forceinline__ double trial_entry(const SysDev &S, int a, int b, con
     const float r2f = fx * fx + fy * fy + fz * fz;
     if (!(r2f < P.rc2f) || r2f == 0.0f) return 0.0;
     const int lj = meta_lip(pj.w), kjl = meta_k(pj.w);
-    near(lj);
     const bool chj = (lj == a || lj == b) && ((sm.m >> kjl) & 1);
     if (chj && lj * P.bpl + kjl < sm.chg_id[ci]) return 0.0;   // a changed pair once, by the lower id
     const double ex = (double)ix * P.qs[0], ey = (double)iy * P.qs[1], ez = (double)iz * P.qs[2];
@@ -210,7 +208,7 @@ __device__ inline void trial_nl_part(const SysDev &S, int p, int par, const Grp 
     const int total = sm.it_beg[nc * G];
     double acc = 0.0;
     for (int f = p + TRIAL_PARTS * t; f < total; f += TRIAL_PARTS * GRP)
-        acc += trial_entry<G>(S, a, b, cur, sm, f, [&](int k) { if (mark) mark_item(k); }, [](int) {});
+        acc += trial_entry<G>(S, a, b, cur, sm, f, [&](int k) { if (mark) mark_item(k); });
     const double part = group_sum(acc, g, sm.sh);   // (its barriers order the group's marks)
     if (t == 0 && mark) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" :: "l"(&C.mark_seq) : "memory");
     if (t == 0) {

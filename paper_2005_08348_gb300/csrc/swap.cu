@@ -22,14 +22,10 @@ namespace mdas {
 // by the lower id only.  Candidates are culled in FP32 from exact integer
 // separations (those within float rounding of rc are decided in FP64); the
 // energies are FP64.  Types come from a functor of (meta, id) and a predicate
-// telling whether a neighbour is changed.  Of the cell's beads, those at first,
-// first + stride, ...; near(lipid) is called for every one inside the cutoff.
-struct NearNone {
-    __device__ void operator()(int) const {}
-};
-template <class NewT, class Changed, class Near = NearNone>
+// telling whether a neighbour is changed.
+template <class NewT, class Changed>
 __device__ double bead_delta(const SysDev &S, const Params &P, int i, uint4 pi, int old_i, int new_i, int slot,
-                             NewT newt, Changed changed, int first = 0, int stride = 1, Near near = Near()) {
+                             NewT newt, Changed changed) {
     const int nx = P.nc[0], ny = P.nc[1], nz = P.nc[2];
     const int cx = (int)(((unsigned long long)pi.x * (unsigned)nx) >> 32);
     const int cy = (int)(((unsigned long long)pi.y * (unsigned)ny) >> 32);
@@ -41,7 +37,7 @@ __device__ double bead_delta(const SysDev &S, const Params &P, int i, uint4 pi, 
     const uint32_t em = P.excl[ki];
     double acc = 0.0;
     const int e = cj * P.capc + S.cell_n[cj];
-    for (int p = cj * P.capc + first; p < e; p += stride) {
+    for (int p = cj * P.capc; p < e; ++p) {
         const uint4 pj = __ldcg(&S.spos[p]);
         const int ix = (int)(pi.x - pj.x), iy = (int)(pi.y - pj.y), iz = (int)(pi.z - pj.z);
         const float fx = (float)ix * P.qsf[0], fy = (float)iy * P.qsf[1], fz = (float)iz * P.qsf[2];
@@ -49,7 +45,6 @@ __device__ double bead_delta(const SysDev &S, const Params &P, int i, uint4 pi, 
         if (!(r2f < P.rc2f) || r2f == 0.0f) continue;
         const int j = S.sorted_id[p];
         if (j == i) continue;
-        near(meta_lip(pj.w));
         const bool chj = changed(pj.w, j);
         if (chj && j < i) continue;
         if (li >= 0 && meta_lip(pj.w) == li && ((em >> meta_k(pj.w)) & 1u)) continue;
@@ -567,14 +562,14 @@ void launch_delta_energy(const LaunchCtx &L, int n) {
 //     chunk whose acceptance would change it (a bit per trial);
 //   k_chain_walk: one cluster of blocks per system decides the trials in order;
 //     one whose bits meet an accepted trial is evaluated again, by the whole
-//     cluster (the FP64 pair terms bound a single SM: about 500 of them at 45
-//     operations, two per clock).
+//     cluster (the FP64 pair terms bound a single SM: some 1300 of them for an
+//     exchange at 28 operations, two per clock).
 // dE is one fixed sum of CHAIN_SLOTS slots, whichever kernel computes it, so
 // the records do not depend on the chunks.
 //
-// Measured, a call of 256 trials: exchanges on a 1424-lipid bilayer 566 us (a
-// launch per trial: 2574), mutations on a 4608-lipid bilayer 482 us (one block
-// for all of them: 11207).
+// Measured, a call of 256 trials: exchanges on a 1424-lipid bilayer 529 us (a
+// launch per trial: 2577), mutations on a 4608-lipid bilayer 348 us (one block
+// for all of them: 10971).
 //
 // Mutation trial T draws Philox (0, T, TAG_MUTATE, 0): lipid a from word 0, the
 // new type among the other n_lt - 1 types from word 1, u from words 2-3; accept
@@ -629,30 +624,127 @@ __device__ __forceinline__ void chain_setup(const SysDev &S, const ChainProp &pr
     }
 }
 
-// Slot `slot` of the dE of the trial in sm: its entries slot, slot +
-// CHAIN_SLOTS, ...  (a mutation's entry: every fourth bead of one of a changed
-// bead's 27 cells)
+// One lane's part of the dE of the trial in sm: the warp's entries are those of
+// slots slot0 .. slot0 + 31, of every CHAIN_SLOTS.  An exchange's entry is a list
+// entry of a changed bead; a mutation's is every fourth bead of one of a changed
+// bead's 27 cells.  ring: 64 entries of this warp.
+//
+// The FP64 pipe (two operations per clock and SM, whole warps) bounds it, and
+// less than half of a list's entries and a sixth of the cells' beads are inside
+// the cutoff: the warp culls in FP32, lets the survivors wait in the ring and
+// takes 32 at a time through FP64, and it fetches four rounds of entries at a
+// time: 256 exchange trials at 1424 lipids 610 to 529 us, 256 mutation trials at
+// 4608 lipids 433 to 348 (each lane with its own entries, one after another).
 template <int G, class Near>
-__device__ __forceinline__ double chain_slot(const SysDev &S, const ChainProp &pr, const uint4 *cur, const TrialSmem &sm,
-                                             int slot, Near near) {
+__device__ __forceinline__ double chain_warp(const SysDev &S, const ChainProp &pr, const uint4 *cur, const TrialSmem &sm,
+                                             int slot0, int lane, int4 *ring, Near near) {
+    constexpr unsigned FULL = 0xffffffffu;
+    constexpr int ROUNDS = 4;
     const Params &P = *S.p;
+    const float q0 = P.qsf[0], q1 = P.qsf[1], q2 = P.qsf[2];
     double acc = 0.0;
+    int head = 0, tail = 0;
+    auto take = [&](int nt) {
+        if (lane < nt) {
+            const int4 e = ring[(head + lane) & 63];
+            const double ex = (double)e.x * P.qs[0], ey = (double)e.y * P.qs[1], ez = (double)e.z * P.qs[2];
+            const float fx = (float)e.x * q0, fy = (float)e.y * q1, fz = (float)e.z * q2;
+            const double r2 = fma(ex, ex, fma(ey, ey, ez * ez));
+            const float r2f = fx * fx + fy * fy + fz * fz;
+            if (inside_rc(P, r2, r2f))
+                acc += pair_du(P, e.w & 15, (e.w >> 4) & 15, (e.w >> 8) & 15, (e.w >> 12) & 15, r2, r2f);
+        }
+        head += nt;
+        __syncwarp();
+    };
+    // a candidate pj (v: there is one) of bead pi; types(): its old and new
+    // types, or a negative number when the pair does not count
+    auto offer = [&](bool v, uint4 pi, uint4 pj, auto types) {
+        const int ix = (int)(pi.x - pj.x), iy = (int)(pi.y - pj.y), iz = (int)(pi.z - pj.z);
+        const float fx = (float)ix * q0, fy = (float)iy * q1, fz = (float)iz * q2;
+        const float r2f = fx * fx + fy * fy + fz * fz;
+        int ty = -1;
+        if (v && r2f < P.rc2f && r2f != 0.0f) ty = types();
+        const unsigned bal = __ballot_sync(FULL, ty >= 0);
+        if (ty >= 0) ring[(tail + __popc(bal & ((1u << lane) - 1u))) & 63] = make_int4(ix, iy, iz, ty);
+        tail += __popc(bal);
+        __syncwarp();
+        if (tail - head >= 32) take(32);
+    };
     if constexpr (G > 0) {
-        const int total = sm.it_beg[sm.nchg * G];
-        for (int f = slot; f < total; f += CHAIN_SLOTS)
-            acc += trial_entry<G>(S, pr.a, pr.b, cur, sm, f, [](int) {}, near);
+        const int a = pr.a, b = pr.b, cols = sm.nchg * G, total = sm.it_beg[cols];
+        for (int f0 = slot0; f0 < total; f0 += ROUNDS * CHAIN_SLOTS) {
+            int ci[ROUNDS], kj[ROUNDS];
+            uint4 pj[ROUNDS];
+#pragma unroll
+            for (int u = 0; u < ROUNDS; ++u) {
+                const int f = f0 + u * CHAIN_SLOTS + lane;
+                int lo = 0, hi = cols - 1;        // the (bead, column) holding entry f
+                while (lo < hi) {
+                    const int mid = (lo + hi + 1) >> 1;
+                    if (sm.it_beg[mid] <= f) lo = mid; else hi = mid - 1;
+                }
+                ci[u] = lo / G;
+                kj[u] = f < total ? S.nl[nl_at<G>(P.npad, sm.chg_k[ci[u]], f - sm.it_beg[lo], lo % G)] : -1;
+            }
+#pragma unroll
+            for (int u = 0; u < ROUNDS; ++u)
+                pj[u] = kj[u] >= 0 ? __ldcg(cur + MDAS_IDX(*S.c, kj[u], P.n)) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+            for (int u = 0; u < ROUNDS; ++u) {
+                if (f0 + u * CHAIN_SLOTS >= total) break;
+                const int c = ci[u];
+                offer(kj[u] >= 0, sm.chg_pos[c], pj[u], [&]() {
+                    const int l = meta_lip(pj[u].w), k = meta_k(pj[u].w);
+                    near(l);
+                    const bool ch = (l == a || l == b) && ((sm.m >> k) & 1);
+                    if (ch && l * P.bpl + k < sm.chg_id[c]) return -1;     // a changed pair once, by the lower id
+                    const int oj = meta_ta(pj[u].w);
+                    const int nj = ch ? (int)P.lbt[(l == a ? sm.tb : sm.ta) * 16 + k] : oj;
+                    return sm.chg_old[c] | oj << 4 | sm.chg_new[c] << 8 | nj << 12;
+                });
+            }
+        }
     } else {
-        const int a = pr.a, ta = sm.ta, tn = sm.tb;
-        auto changed = [&](uint32_t mj, int) {
-            return meta_lip(mj) == a && P.lbt[ta * 16 + meta_k(mj)] != P.lbt[tn * 16 + meta_k(mj)];
-        };
-        auto newt = [&](uint32_t mj, int) { return (int)P.lbt[tn * 16 + meta_k(mj)]; };
-        for (int f = slot; f < sm.nchg * 27 * 4; f += CHAIN_SLOTS) {
-            const int ci = f / 108, q = f % 108;
-            acc += bead_delta(S, P, sm.chg_id[ci], sm.chg_pos[ci], sm.chg_old[ci], sm.chg_new[ci], q / 4, newt, changed,
-                              q % 4, 4, near);
+        const int a = pr.a, ta = sm.ta, tn = sm.tb, total = sm.nchg * 27 * 4;
+        const int nx = P.nc[0], ny = P.nc[1], nz = P.nc[2];
+        for (int f0 = slot0; f0 < total; f0 += CHAIN_SLOTS) {
+            const int f = f0 + lane, ci = f < total ? f / 108 : 0, q = f % 108, o = q >> 2;
+            const uint4 pi = sm.chg_pos[ci];
+            int x = (int)(((unsigned long long)pi.x * (unsigned)nx) >> 32) + o % 3 - 1;
+            int y = (int)(((unsigned long long)pi.y * (unsigned)ny) >> 32) + (o / 3) % 3 - 1;
+            int z = (int)(((unsigned long long)pi.z * (unsigned)nz) >> 32) + o / 9 - 1;
+            x += x < 0 ? nx : (x >= nx ? -nx : 0);
+            y += y < 0 ? ny : (y >= ny ? -ny : 0);
+            z += z < 0 ? nz : (z >= nz ? -nz : 0);
+            const int cj = (z * ny + y) * nx + x, e = f < total ? S.cell_n[cj] : 0, i = sm.chg_id[ci];
+            const int ki = meta_k(pi.w);
+            const uint32_t em = P.excl[ki];
+            const uint4 *sp = S.spos + (size_t)cj * P.capc;
+            for (int p0 = q & 3; __any_sync(FULL, p0 < e); p0 += 4 * ROUNDS) {
+                uint4 pj[ROUNDS];
+#pragma unroll
+                for (int u = 0; u < ROUNDS; ++u)
+                    pj[u] = p0 + 4 * u < e ? __ldcg(sp + p0 + 4 * u) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+                for (int u = 0; u < ROUNDS; ++u) {
+                    if (!__any_sync(FULL, p0 + 4 * u < e)) break;
+                    offer(p0 + 4 * u < e, pi, pj[u], [&]() {
+                        const int l = meta_lip(pj[u].w), k = meta_k(pj[u].w);
+                        if (l == a && k == ki) return -1;                  // the bead itself
+                        near(l);
+                        const int old = meta_ta(pj[u].w);
+                        const int nj = l == a ? (int)P.lbt[tn * 16 + k] : old;
+                        const bool ch = l == a && P.lbt[ta * 16 + k] != P.lbt[tn * 16 + k];
+                        if (ch && l * P.bpl + k < i) return -1;            // a changed pair once, by the lower id
+                        if (l == a && ((em >> k) & 1u)) return -1;         // bonded
+                        return sm.chg_old[ci] | old << 4 | sm.chg_new[ci] << 8 | (ch ? nj : old) << 12;
+                    });
+                }
+            }
         }
     }
+    if (tail != head) take(tail - head);
     return acc;
 }
 
@@ -660,6 +752,16 @@ __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
     return v;                                  // lane 0
+}
+
+// The sum of the warp sums, on every lane of a warp (a fixed tree: one after
+// another they took as long as the cutoff tests).
+__device__ __forceinline__ double chain_total(const double *sums, int lane) {
+    static_assert(CHAIN_SUMS == 32, "a warp sum per lane");
+    double v = sums[lane];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
 }
 
 // grid (1, n_sys): node 2 t + side + 1 of trial t enters the list of the lipid
@@ -681,6 +783,7 @@ __global__ void __launch_bounds__(CHAIN_THREADS) k_chain_eval(const SysDev *__re
     const Params &P = *S.p;
     __shared__ TrialSmem sm;
     __shared__ double sums[CHAIN_SUMS];
+    __shared__ int4 ring[CHAIN_THREADS / 32][64];
     __shared__ unsigned bits[CHAIN_WORDS];
     const int t = blockIdx.x, x = threadIdx.x, lane = x & 31;
     const ChainProp pr = chain_draw<G>(P, S.c->trial + (unsigned long long)t);
@@ -698,16 +801,17 @@ __global__ void __launch_bounds__(CHAIN_THREADS) k_chain_eval(const SysDev *__re
     };
     if (x < 2) meets(x ? pr.b : pr.a);
     for (int i = 0; i < CHAIN_BLOCKS; ++i) {
-        const double s = warp_sum(chain_slot<G>(S, pr, cur, sm, CHAIN_THREADS * i + x, meets));
+        const double s = warp_sum(chain_warp<G>(S, pr, cur, sm, CHAIN_THREADS * i + (x & ~31), lane, ring[x >> 5], meets));
         if (lane == 0) sums[(CHAIN_THREADS / 32) * i + (x >> 5)] = s;
     }
     __syncthreads();
     if (x < CHAIN_WORDS) S.conflict[t * CHAIN_WORDS + x] = bits[x];
-    if (x == 0) {
-        double dE = 0.0;
-        for (int i = 0; i < CHAIN_SUMS; ++i) dE += sums[i];
-        S.tdE[t] = dE;
-        S.tprop[t] = make_int4(pr.a, pr.b, sm.ta, sm.tb);
+    if (x < 32) {
+        const double dE = chain_total(sums, lane);
+        if (lane == 0) {
+            S.tdE[t] = dE;
+            S.tprop[t] = make_int4(pr.a, pr.b, sm.ta, sm.tb);
+        }
     }
 }
 
@@ -732,6 +836,7 @@ k_chain_walk(const SysDev *__restrict__ sys, int m, int spec) {
     Counters &C = *S.c;
     __shared__ TrialSmem sm;
     __shared__ double sums[CHAIN_SUMS];
+    __shared__ int4 ring[CHAIN_THREADS / 32][64];
     __shared__ int cmd;
     __shared__ unsigned bits[CHAIN_MAX * CHAIN_WORDS];
     const int x = threadIdx.x, lane = x & 31;
@@ -777,8 +882,7 @@ k_chain_walk(const SysDev *__restrict__ sys, int m, int spec) {
                 double dE = __shfl_sync(0xffffffffu, mine_dE, src);
                 int ta = __shfl_sync(0xffffffffu, mine_ta, src), tb = __shfl_sync(0xffffffffu, mine_tb, src);
                 if (fresh) {
-                    dE = 0.0;
-                    for (int i = 0; i < CHAIN_SUMS; ++i) dE += sums[i];
+                    dE = chain_total(sums, lane);
                     ta = sm.ta;
                     tb = sm.tb;
                     fresh = false;
@@ -818,7 +922,8 @@ k_chain_walk(const SysDev *__restrict__ sys, int m, int spec) {
         const ChainProp pr = chain_draw<G>(P, T0 + (unsigned long long)todo);
         if (x < 32) chain_setup<G>(S, pr, cur, lane, sm);
         __syncthreads();
-        const double s = warp_sum(chain_slot<G>(S, pr, cur, sm, CHAIN_THREADS * rank + x, [](int) {}));
+        const double s = warp_sum(chain_warp<G>(S, pr, cur, sm, CHAIN_THREADS * rank + (x & ~31), lane, ring[x >> 5],
+                                                [](int) {}));
         if (lane == 0)
             asm volatile("st.shared::cluster.f64 [%0], %1;"
                          :: "r"(cluster_addr(&sums[(CHAIN_THREADS / 32) * rank + (x >> 5)], 0)), "d"(s) : "memory");
