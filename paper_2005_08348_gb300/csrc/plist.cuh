@@ -47,7 +47,8 @@
 // list rebuilds, thermostat, exchange trials) with grid-wide barriers
 // between the phases instead of kernel launches.  When the step items leave
 // groups free, each step runs beside the previous step's close and exchange
-// trial, one grid barrier per step.
+// trial, one grid barrier per step; otherwise beside its close where no trial
+// follows.
 #pragma once
 #include <algorithm>
 #include <cmath>
