@@ -631,7 +631,8 @@ __global__ void __launch_bounds__(BEAD_BLOCK) k_bonded_energy(const SysDev *__re
 // The FP64 pipe bounds it (two operations per clock and SM): each pair goes
 // through it once, at about 20 operations with 1/r from rsqrt_near, where the force
 // kernel's pass took every pair twice with a square root, a division and the
-// forces (a call for forces and energies, 1152 lipids: 654 to 334 us).
+// forces (a call for forces and energies, 1152 lipids: 654 to 334 us, and 275
+// with rsqrt_near and fewer launches and copies).
 constexpr int ENERGY_WARPS = 4;
 __global__ void __launch_bounds__(32 * ENERGY_WARPS) k_cell_energy(const SysDev *__restrict__ sys,
                                                                    const int2 *__restrict__ bmap, int n_items) {
