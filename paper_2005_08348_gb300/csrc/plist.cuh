@@ -526,11 +526,14 @@ __device__ void nl_build_dealt(const SysDev *sys, int n_sys, int gw, int nw, int
 }
 
 // Four list entries: read once per step, so they skip L1 (which keeps the
-// positions and tables the step reuses)
+// positions and tables the step reuses).  Not a non-coherent load (.nc): a
+// launch writes the lists again at every build, and only data that no one
+// writes during a kernel may be read that way; this one is ordered by the
+// build's barriers like any other.
 __device__ __forceinline__ int4 ld_list(const int4 *p) {
     int4 v;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.b32 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    asm volatile("ld.global.L1::no_allocate.v4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
     return v;
 }
 
