@@ -820,8 +820,10 @@ __device__ __forceinline__ unsigned cluster_addr(const void *p, unsigned rank) {
     asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((unsigned)__cvta_generic_to_shared(p)), "r"(rank));
     return r;
 }
+// (not the .aligned forms: those want the whole warp to arrive together, and
+// the code before it diverges by lane)
 __device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
 }
 
 // grid (CHAIN_BLOCKS, n_sys), one cluster per system: trials 0 .. m - 1 of the

@@ -24,3 +24,10 @@ def test_no_non_coherent_load():
     a line from before a list build, whatever barrier lies between."""
     for name, txt in _sources().items():
         assert not re.search(r"ld\.global(\.\w+|::\w+)*\.nc\b|\b__ldg\s*\(", txt), name
+
+
+def test_no_aligned_cluster_barrier():
+    """k_chain_walk comes to its cluster barriers from code that diverges by
+    lane, where an .aligned arrival is undefined (it may wait without end)."""
+    for name, txt in _sources().items():
+        assert not re.search(r"barrier\.cluster\.(arrive|wait)(\.\w+)*\.aligned", txt), name
