@@ -170,8 +170,8 @@ __device__ void thermostat_block(const SysDev &S, const Params &P) {
 }
 
 // Before an MD segment of n steps: grid (blocks of variates + 1, n_sys).  The
-// last block of a system sets the factor of its first step (thermostat_block);
-// the others draw the variates of the segment, a warp of 32 each: two groups,
+// last block of a system sets the factor of its first step (thermostat_block)
+// and clears the trials' marks; the others draw the variates of the segment, a warp of 32 each: two groups,
 // and R1 and S of a step apart.  The variates are FP64 logarithms, roots and a
 // cosine, which the FP64 pipe (two operations per clock and SM) bounds: a warp
 // per SM.  One launch, both parts beside each other, where two kernels went one
@@ -184,6 +184,10 @@ __global__ void __launch_bounds__(THERMO_THREADS) k_thermo(const SysDev *__restr
     const Params &P = *S.p;
     Counters &C = *S.c;
     if (blockIdx.x + 1 == gridDim.x) {
+        // no marks of trials before the segment: the trials between two
+        // segments move the counter on, and with it the parity of a trial's
+        // bitmap, and mark and clear nothing
+        for (int x = threadIdx.x; x < 2 * P.mark_words; x += blockDim.x) S.tmark[x] = 0u;
         thermostat_block<Real>(S, P);
         return;
     }

@@ -187,7 +187,8 @@ __device__ __forceinline__ double trial_entry(const SysDev &S, int a, int b, con
 // changed bead or one of its list partners, then count themselves in
 // mark_seq; the decision is published by the trial counter only after the
 // exchange is applied.  Every trial clears the other bitmap for the next one
-// (its last readers finished before this trial started).
+// (its last readers finished before this trial started); both are clear when an
+// MD segment starts (k_thermo).
 template <int G>
 __device__ inline void trial_nl_part(const SysDev &S, int p, int par, const Grp &g, TrialSmem &sm, bool mark) {
     constexpr int NL_BEADS = NL_BLOCK / G;
