@@ -463,8 +463,8 @@ mdas_status mdas_pair_kernel_time(mdas_system *s, double *total_ms, int64_t *lau
 
 /* Per-system counters: MD steps, force evaluations (one per MD step and one
  * per exchange trial, as counted in Sec. 3), trials, null and accepted trials,
- * MDAS moves and accepted moves, and the kernel launches of replayed CUDA
- * graphs that advanced the system. */
+ * MDAS moves and accepted moves, and the kernel launches of MD segments and
+ * mutation trials that advanced the system. */
 typedef struct {
     int64_t md_steps, force_evals, trials, null_trials, accepted, moves, moves_accepted, kernel_launches;
     int64_t list_builds;               /* pair-list builds of the MD step */

@@ -121,7 +121,7 @@ struct mdas_system {
     int trial_path = MDAS_TRIALS_AUTO;   // mdas_set_trial_path
     double pair_ms = 0.0;
     long long pair_launches = 0;
-    long long kernel_launches = 0;   // kernel launches (graph kernel nodes included) that advanced this system
+    long long kernel_launches = 0;   // kernel launches of MD segments and mutation trials that advanced this system
 };
 
 namespace {
@@ -1102,8 +1102,7 @@ mdas_status mdas_mutation_trials(mdas_system *s, int32_t n_trials, const double 
     mdas_status st = build_cells(s, b);
     if (st != MDAS_OK) return st;
     LaunchCtx L = b.ctx();
-    launch_mutation_trials(L, n_trials, s->n_lip);
-    s->kernel_launches += 1;
+    s->kernel_launches += launch_mutation_trials(L, n_trials, s->n_lip);
     Counters c1;
     CK(cudaMemcpyAsync(&c1, s->hs.c, sizeof(Counters), cudaMemcpyDeviceToHost, s->stream));
     CK(cudaStreamSynchronize(s->stream));

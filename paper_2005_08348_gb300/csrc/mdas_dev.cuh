@@ -409,7 +409,8 @@ void launch_snapshot(const LaunchCtx &L);
 void launch_delta_energy(const LaunchCtx &L, int n_changed_lipids);
 // n trials of every system in order, many per launch; max_lip: lipids of the largest system
 void launch_swap_trials(const LaunchCtx &L, int n, int max_lip);       // over the pair lists (valid lists)
-void launch_mutation_trials(const LaunchCtx &L, int n, int max_lip);   // over the cells (a current cell list)
+int launch_mutation_trials(const LaunchCtx &L, int n, int max_lip);    // over the cells (a current cell list);
+                                                                       // returns its launches
 // the work term of the lambda step l0 -> l1 from the pair list (valid lists)
 void launch_mdas_dE_nl(const LaunchCtx &L, double l0, double l1, double dlambda);
 void launch_head_rdf(const SysDev *dsys, int n_lip, int lt_sel, int head_k, double r_max, int n_bins, uint4 *info,

@@ -954,19 +954,23 @@ k_chain_walk(const SysDev *__restrict__ sys, int m, int spec) {
 // has some 25 lipids in reach, so a chunk of n_lip / 16 evaluates about one
 // trial in five again.  From CHAIN_MIN trials on (shorter chunks of small
 // bilayers, where most trials meet, are walked without the first evaluation).
+// Returns the number of launches.
 template <int G>
-static void chain_launch(const LaunchCtx &L, int n, int max_lip) {
+static int chain_launch(const LaunchCtx &L, int n, int max_lip) {
+    int launches = 0;
     const int chunk = max_lip / 16 >= CHAIN_MAX ? CHAIN_MAX : max_lip / 16;
     const int spec = chunk >= CHAIN_MIN && n >= CHAIN_MIN;
     const int step = spec ? chunk : CHAIN_MAX;
     for (int done = 0; done < n; done += step) {
         const int m = n - done < step ? n - done : step;
+        launches += spec ? 3 : 1;
         if (spec) {
             k_chain_propose<G><<<dim3(1, L.n_sys), CHAIN_MAX, 0, L.stream>>>(L.sys, m);
             k_chain_eval<G><<<dim3(m, L.n_sys), CHAIN_THREADS, 0, L.stream>>>(L.sys);
         }
         k_chain_walk<G><<<dim3(CHAIN_BLOCKS, L.n_sys), CHAIN_THREADS, 0, L.stream>>>(L.sys, m, spec);
     }
+    return launches;
 }
 
 void launch_swap_trials(const LaunchCtx &L, int n, int max_lip) {
@@ -974,7 +978,7 @@ void launch_swap_trials(const LaunchCtx &L, int n, int max_lip) {
     else chain_launch<4>(L, n, max_lip);
 }
 
-void launch_mutation_trials(const LaunchCtx &L, int n, int max_lip) { chain_launch<0>(L, n, max_lip); }
+int launch_mutation_trials(const LaunchCtx &L, int n, int max_lip) { return chain_launch<0>(L, n, max_lip); }
 
 // ----------------------------------------------------------------- Philox
 __global__ void k_philox(uint32_t k0, uint32_t k1, uint32_t c1, uint32_t c2, uint32_t c3, int n, uint4 *out) {
