@@ -6,10 +6,12 @@
 
 namespace mdas {
 
-// 1/sqrt(r2) in FP64 from a float r2f near r2 (relative difference below
-// 2^-21): the float function's value, widened by its bits, and one third-order
-// step, y (1 + e/2 + 3 e^2/8) with e = 1 - r2 y^2 below 2^-19 (what it leaves out
-// is below 2^-58): within an ulp of FP64, as the square root and the division.
+// 1/sqrt(r2) in FP64 from a float r2f near r2 (the same sum of squares from
+// float offsets: 6 2^-24 at most on each square and 3 more from the sum, a
+// relative difference below 2^-20): the float function's value, widened by its
+// bits, and one third-order step, the binomial series of (1 - e)^(-1/2), y (1 +
+// e/2 + 3 e^2/8) with e = 1 - r2 y^2 below 2^-19 (what it leaves out is below
+// 2^-58): within an ulp of FP64, as the square root and the division.
 // The FP64 pipe takes two operations per clock and SM and bounds every sum over
 // pairs in FP64; this takes five of them, two Newton steps and the conversions
 // to and from float took ten: 20 FP64 steps at 128 lipids 996 to 895 us, 256
