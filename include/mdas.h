@@ -142,8 +142,11 @@ typedef struct {
      * restore).  The pair list is built at earlier positions than the current
      * ones and the thermostat reads the kinetic energy the last MD step left in
      * fixed point; with both carried, MD resumed from a saved state repeats
-     * the uninterrupted run bit for bit (exchange trials counted from the
-     * start of each call: resume at a multiple of swap_every). */
+     * the uninterrupted run of the same calls bit for bit (exchange trials
+     * counted from the start of each call: resume at a multiple of swap_every;
+     * the thermostat factor of a call's first step is computed apart from the
+     * later ones and may differ from what they would be in the last place, so
+     * other lengths of the calls may give other last bits). */
     uint32_t *list_ref;                /* [n*3] fixed-point positions the pair list was built at, bead id order, or NULL */
     int32_t list_valid;                /* get_state: 1 when list_ref was filled (else the list is rebuilt at the next
                                         * MD step); set_state: rebuild the list at list_ref instead */

@@ -171,12 +171,13 @@ __device__ void thermostat_block(const SysDev &S, const Params &P) {
 
 // Before an MD segment of n steps: grid (blocks of variates + 1, n_sys).  The
 // last block of a system sets the factor of its first step (thermostat_block)
-// and clears the trials' marks; the others draw the variates of the segment, a warp of 32 each: two groups,
-// and R1 and S of a step apart.  The variates are FP64 logarithms, roots and a
-// cosine, which the FP64 pipe (two operations per clock and SM) bounds: a warp
-// per SM.  One launch, both parts beside each other, where two kernels went one
-// after the other: with the ending merged too, calls of 20 steps are 1 to 3%
-// shorter and 64 mutation trials took 332 us for 400.
+// and clears the trials' marks; the others draw the variates of the segment, a
+// warp of 32 each: two groups, and R1 and S of a step apart.  The variates are
+// FP64 logarithms, roots and a cosine, which the FP64 pipe (two operations per
+// clock and SM) bounds: a warp per SM.  One launch, both parts beside each
+// other, where two kernels went one after the other: with the ending merged
+// too, calls of 20 steps are 1 to 3% shorter, and 64 mutation trials, whose cell
+// build carried a factor of its own, took 332 us for 400.
 constexpr int THERMO_THREADS = 1024;
 template <typename Real>
 __global__ void __launch_bounds__(THERMO_THREADS) k_thermo(const SysDev *__restrict__ sys, int n) {

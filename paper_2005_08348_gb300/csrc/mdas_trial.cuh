@@ -14,9 +14,9 @@ namespace mdas {
 // 2^-58): within an ulp of FP64, as the square root and the division.
 // The FP64 pipe takes two operations per clock and SM and bounds every sum over
 // pairs in FP64; this takes five of them, two Newton steps and the conversions
-// to and from float took ten: 20 FP64 steps at 128 lipids 996 to 895 us, 256
-// exchange trials at 1424 lipids 537 to 501, 20 FP32 steps with a trial each at
-// 1152 lipids 571 to 561.
+// to and from float took ten: 20 FP64 steps at 128 lipids 996 to 895 us, 20 FP32
+// steps with a trial each at 1152 lipids 571 to 561, 256 exchange trials at 1424
+// lipids 7% less.
 __device__ __forceinline__ double rsqrt_near(double r2, float r2f) {
     const unsigned b = __float_as_uint(rsqrtf(r2f));          // positive and normal
     const double y = __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));

@@ -223,7 +223,8 @@ __device__ void set_lipid_type(const SysDev &S, const Params &P, int l, int lt) 
 }
 
 
-// One exchange trial per system from the pair list: grid (TRIAL_PARTS, n_sys).
+// One exchange trial per system from the pair list, after a step of the separate
+// launches: grid (TRIAL_PARTS, n_sys).
 template <int G>
 __global__ void __launch_bounds__(GRP) k_trial_nl(const SysDev *__restrict__ sys) {
     __shared__ TrialSmem sm;
@@ -567,9 +568,10 @@ void launch_delta_energy(const LaunchCtx &L, int n) {
 // dE is one fixed sum of CHAIN_SLOTS slots, whichever kernel computes it, so
 // the records do not depend on the chunks.
 //
-// Measured, a call of 256 trials: exchanges on a 1424-lipid bilayer 529 us (a
-// launch per trial: 2577), mutations on a 4608-lipid bilayer 348 us (one block
-// for all of them: 10971).
+// Measured, a call of 256 trials: exchanges on a 1424-lipid bilayer 530 to 630 us
+// by state and session (a launch per trial: 2580), mutations on a 4608-lipid
+// bilayer 350 to 435 us (one block for all of them: 10970); the same call again
+// and again on one state 473 and 281 us.
 //
 // Mutation trial T draws Philox (0, T, TAG_MUTATE, 0): lipid a from word 0, the
 // new type among the other n_lt - 1 types from word 1, u from words 2-3; accept
@@ -633,8 +635,8 @@ __device__ __forceinline__ void chain_setup(const SysDev &S, const ChainProp &pr
 // less than half of a list's entries and a sixth of the cells' beads are inside
 // the cutoff: the warp culls in FP32, lets the survivors wait in the ring and
 // takes 32 at a time through FP64, and it fetches four rounds of entries at a
-// time: 256 exchange trials at 1424 lipids 610 to 529 us, 256 mutation trials at
-// 4608 lipids 433 to 348 (each lane with its own entries, one after another).
+// time: 256 exchange trials at 1424 lipids 13% less, 256 mutation trials at 4608
+// lipids 20% less than each lane with its own entries, one after another.
 template <int G, class Near>
 __device__ __forceinline__ double chain_warp(const SysDev &S, const ChainProp &pr, const uint4 *cur, const TrialSmem &sm,
                                              int slot0, int lane, int4 *ring, Near near) {
