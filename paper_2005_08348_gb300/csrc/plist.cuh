@@ -750,11 +750,13 @@ __device__ __forceinline__ void nl_step_item(int k0, int par, int *viol, const G
     // the separations are known, and the index registers the group after, so
     // every load has most of a group to arrive.
     //
-    // What bounds the loop: the wavefronts of its gathers and table reads (about
-    // 22 per warp and row before, 14 of them the gather) and, next, its
-    // instructions (72 per entry before).  With 8-byte table entries, four
-    // indices per load, no branch per pair and no bounds test per row a step of
-    // the 1152-lipid bilayer takes 14.8 us without a trial (17.5 before), of
+    // What bounds the loop: the wavefronts of its gathers and table reads and,
+    // next, its instructions.  With 8-byte table entries, four indices per
+    // load, no branch per pair and no bounds test per row, the step as a kernel
+    // of its own takes 23.4 wavefronts of the L1 data pipe per warp and list row
+    // (24.9 before; 15.3 of them global, 17.6 before) and 81 lane slots of
+    // instructions per list entry (93 before); in the persistent kernel a step
+    // of the 1152-lipid bilayer takes 14.8 us without a trial (17.5 before), of
     // the 4608-lipid one 46.8 (54), of the 128-lipid one 8.6 (12.2).
     const int rows = cnt;
     unsigned long long aw = 0;
